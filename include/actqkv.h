@@ -341,7 +341,8 @@ int actqkv_append_window(const actqkv_config* cfg, const actqkv_batch* batch, co
  * Enqueues, in this order and with the same results, actqkv_bias_probe (when update_probe is non-zero),
  * actqkv_score_select, actqkv_retrieval_attention, actqkv_append_window and, when next_positions (HOST array of
  * n_next sequences) is given, actqkv_set_positions.  The struct holds the arguments of those calls under their
- * names; what may be NULL there may be NULL here.  Returns the first error; the stages before it are enqueued. */
+ * names; what may be NULL there may be NULL here.  n_next must be the batch's number of sequences (ACTQKV_ERR_SHAPE, nothing
+ * is enqueued).  Returns the first error of a stage; the stages before it are enqueued. */
 typedef struct actqkv_step_buffers {
   const void *q, *k_win, *v_win;
   void* out;

@@ -152,6 +152,9 @@ def n_candidates(cfg: Config, p0: int) -> int:
 def set_positions(cfg, positions, pos0, n_cand=None, stream=None):
     """pos0[i] = positions[i] (host integers) and the matching candidate counts, without a copy or a wait."""
     host = array.array("q", positions)
+    for t in (pos0, n_cand):               # the kernel writes one entry per position
+        if t is not None and t.numel() != len(host):
+            raise ActQKVError(f"{len(host)} positions for {t.numel()} sequences")
     _check(_lib.actqkv_set_positions(C.byref(cfg), len(host), host.buffer_info()[0], _ptr(pos0), _ptr(n_cand),
                                      _stream(stream)))
 
@@ -319,9 +322,13 @@ class RetrievalState:
         self.host_pos0 = [0] * n_seq
 
     def set_positions(self, pos0_list):
-        """Host knows where each sequence stands; mirrors it to the device arrays."""
-        self.host_pos0 = [int(p) for p in pos0_list]
-        set_positions(self.cfg, self.host_pos0, self.pos0, self.n_cand)
+        """Host knows where each sequence stands; mirrors it to the device arrays.  A list of one position
+        goes for every sequence."""
+        positions = [int(p) for p in pos0_list]
+        if len(positions) == 1:
+            positions *= self.batch.n_seq
+        set_positions(self.cfg, positions, self.pos0, self.n_cand)
+        self.host_pos0 = positions
 
     def step(self, q, k_win, v_win, out, n_tokens=None, lse=None, fused=True, update_probe=True,
              advance=True, overlap_append=False):
