@@ -327,7 +327,16 @@ class RetrievalState:
         positions = [int(p) for p in pos0_list]
         if len(positions) == 1:
             positions *= self.batch.n_seq
-        set_positions(self.cfg, positions, self.pos0, self.n_cand)
+        if not self.pos0.is_cuda:              # a state kept on the host
+            if len(positions) != self.pos0.numel():
+                raise ActQKVError(f"{len(positions)} positions for {self.pos0.numel()} sequences")
+            self.pos0.copy_(torch.tensor(positions, dtype=torch.int64))
+            self.n_cand.copy_(torch.tensor([n_candidates(self.cfg, p) for p in positions], dtype=torch.int32))
+        elif self.pos0.get_device() == torch.cuda.current_device():
+            set_positions(self.cfg, positions, self.pos0, self.n_cand)
+        else:                                  # the kernel runs where the state lives
+            with torch.cuda.device(self.pos0.device):
+                set_positions(self.cfg, positions, self.pos0, self.n_cand)
         self.host_pos0 = positions
 
     def step(self, q, k_win, v_win, out, n_tokens=None, lse=None, fused=True, update_probe=True,

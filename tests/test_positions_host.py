@@ -1,5 +1,6 @@
 """As many positions as sequences: a list that is longer or shorter is an error before anything is enqueued (the
-kernel writes one entry of pos0 and n_cand per position), a list of one goes for every sequence."""
+kernel writes one entry of pos0 and n_cand per position), a list of one goes for every sequence.  They are set where
+the state lives: in host memory, or by a launch on its own device."""
 import ctypes as C
 
 import pytest
@@ -38,6 +39,49 @@ def test_step_refuses_positions_of_another_number_of_sequences(B, n_seq, n_next)
 
     assert call(n_next) == -3          # ahead of the first stage, which would refuse the NULL buffers
     assert call(n_seq) == -1
+
+
+def test_positions_of_a_state_on_the_host(B):
+    cfg = B.make_config(wl.tiny_pr1())
+    st = B.RetrievalState(cfg, n_seq=3, device="cpu")
+    st.set_positions([10, 700, 3000])
+    assert st.pos0.tolist() == st.host_pos0 == [10, 700, 3000]
+    assert st.n_cand.tolist() == [B.n_candidates(cfg, p) for p in (10, 700, 3000)]
+    st.set_positions([640])
+    assert st.pos0.tolist() == st.host_pos0 == [640] * 3
+    for bad in ([], [1, 2], [1, 2, 3, 4]):
+        with pytest.raises(B.ActQKVError):
+            st.set_positions(bad)
+    assert st.pos0.tolist() == st.host_pos0 == [640] * 3
+
+
+def test_positions_are_set_on_the_device_of_the_state(B, monkeypatch):
+    """Another device is current: the launch goes to the state's own device and its stream."""
+    import contextlib
+    import torch
+    current, seen = [0], []
+
+    @contextlib.contextmanager
+    def device(d):
+        before, current[0] = current[0], torch.device(d).index
+        yield
+        current[0] = before
+
+    class Pos0:
+        is_cuda, device = True, torch.device("cuda:1")
+
+        def get_device(self):
+            return 1
+
+    monkeypatch.setattr(torch.cuda, "device", device)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: current[0])
+    monkeypatch.setattr(B, "set_positions", lambda *args: seen.append((current[0], args[1])))
+    st = B.RetrievalState(B.make_config(wl.tiny_pr1()), n_seq=2, device="cpu")
+    st.pos0 = Pos0()
+    st.set_positions([3, 4])
+    current[0] = 1
+    st.set_positions([5, 6])
+    assert seen == [(1, [3, 4]), (1, [5, 6])] and current[0] == 1
 
 
 @pytest.mark.gpu
