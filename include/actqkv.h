@@ -259,10 +259,10 @@ int actqkv_score_select(const actqkv_config* cfg, const actqkv_batch* batch, con
  * (CTA pairs where they fill the SMs in one wave, else two query tiles per CTA with the key stream cut over a
  * cluster).  Every other type or head size runs on the general fp32-accumulate kernel.
  * Preconditions of the tcgen05 kernels (the general kernel has none of them):
- *  - p0 need not sit on a page boundary, but the rows of the last, partly filled cache page that
- *    lie past p0 must hold finite values: they are masked out of the softmax yet still enter the
- *    P V product with weight 0, and 0 x NaN is NaN.  A zero-initialised pool satisfies this, and
- *    actqkv_append_window zero-fills the rest of the last page it touches.
+ *  - Steps of whole 128-token tiles with an even G, and steps of 33 to 128 rows: p0 need not sit on a page boundary, but
+ *    the rows of the last, partly filled cache page that lie past p0 must hold finite values: they are masked out of
+ *    the softmax yet may still enter the P V product with weight 0, and 0 x NaN is NaN.  A zero-initialised pool
+ *    satisfies this, and actqkv_append_window zero-fills the rest of the last page it touches.
  *  - Steps of whole 128-token tiles with an even G multiply P and V in fp16: |v| <= 65504 (larger finite values
  *    saturate); the others take P as two bf16 terms. */
 int actqkv_retrieval_attention(const actqkv_config* cfg, const actqkv_batch* batch, const void* q,
@@ -283,9 +283,9 @@ int actqkv_retrieval_attention(const actqkv_config* cfg, const actqkv_batch* bat
  *   workspace  device scratch of at least actqkv_decode_workspace_bytes(...) bytes, 16-byte
  *              aligned, caller-owned, contents undefined on entry and exit; may be NULL when
  *              the split count is 1.  Calls that overlap on the GPU need distinct workspaces.
- * The rows of the last, partly filled cache page that lie past p0 must hold finite values
- * (e.g. a zero-initialised pool): they are masked out of the softmax but still enter the
- * P V product with weight 0.
+ * In steps of more than 32 rows the rows of the last, partly filled cache page that lie past p0 must hold finite
+ * values (e.g. a zero-initialised pool): they are masked out of the softmax but still enter the P V product with
+ * weight 0.
  * Returns ACTQKV_ERR_UNSUPPORTED for shapes this kernel does not serve, ACTQKV_ERR_SHAPE when
  * workspace_bytes is too small. */
 int32_t actqkv_decode_splits(const actqkv_config* cfg, const actqkv_batch* batch);

@@ -194,7 +194,7 @@ attention_decode_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
       } else if (j_lo + j < past_tiles) {
         if (lane < 16) tma_load_4d(sbase + half * kSubTileBytes + slot * 2048u, tm_pages, full, half * 64, 0, g, page);
       } else if (lane < 2) {
-        tma_load_3d(sbase + lane * kSubTileBytes, tm_win, full, lane * 64, g, unit * nt);
+        tma_load_4d(sbase + lane * kSubTileBytes, tm_win, full, lane * 64, g, 0, unit);
       }
       issued = j + 1;
       if ((j & 3) == 0) page_next = resolve((j >> 2) + 1);   // after the issue: its stall is behind the ring
@@ -517,12 +517,12 @@ int launch_attention_decode(const actqkv_config* cfg, const Batch& b, const Attn
     const cuuint32_t box[3] = {64, cuuint32_t(G), cuuint32_t(kBM / G)};
     if (!encode(&tm_q, a.q, 3, dims, str, box)) return ACTQKV_ERR_LAUNCH;
   }
-  {
-    const cuuint64_t dims[3] = {cuuint64_t(kD), cuuint64_t(Hkv), cuuint64_t(U) * nt};
-    const cuuint64_t str[2] = {cuuint64_t(kD) * 2, cuuint64_t(Hkv) * kD * 2};
-    const cuuint32_t box[3] = {64, 1, cuuint32_t(kBN)};
-    if (!encode(&tm_kw, a.k_win, 3, dims, str, box)) return ACTQKV_ERR_LAUNCH;
-    if (!encode(&tm_vw, a.v_win, 3, dims, str, box)) return ACTQKV_ERR_LAUNCH;
+  {      // the unit is a dimension of its own: rows of the box behind the unit's tokens are zeros, not its neighbour's
+    const cuuint64_t dims[4] = {cuuint64_t(kD), cuuint64_t(Hkv), cuuint64_t(nt), cuuint64_t(U)};
+    const cuuint64_t str[3] = {cuuint64_t(kD) * 2, cuuint64_t(Hkv) * kD * 2, cuuint64_t(nt) * Hkv * kD * 2};
+    const cuuint32_t box[4] = {64, 1, cuuint32_t(kBN), 1};
+    if (!encode(&tm_kw, a.k_win, 4, dims, str, box)) return ACTQKV_ERR_LAUNCH;
+    if (!encode(&tm_vw, a.v_win, 4, dims, str, box)) return ACTQKV_ERR_LAUNCH;
   }
   {
     const cuuint64_t dims[4] = {cuuint64_t(kD), 16, cuuint64_t(Hkv), cuuint64_t(b.n_layers) * cfg->n_phys_pages};

@@ -314,7 +314,7 @@ attention_decode_t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid
       uint32_t full = 0;
       const uint32_t sbase = claim(a_end, uint32_t(2 * ksteps_new) * 2048u, full);
       if (ok && lane < 2 * ksteps_new && (is_v || a_end != dp.drop_k_tile))
-        tma_load_4d(sbase + lane * 2048u, tm_win, full, 0, unit * nt + lane * 8, 0, g);
+        tma_load_5d(sbase + lane * 2048u, tm_win, full, 0, lane * 8, 0, g, unit);      // (rows behind the unit's last token: zeros)
       __syncwarp();
       if (ok) issued = early;
     }
@@ -373,7 +373,16 @@ attention_decode_t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid
       if (i == early) n_tiles = total_after_wait(false);
       if (i >= n_tiles) break;
       const int pos = 2 * i + 1, s = pos % kRing, j = i * n_ranks + rank;
-      ok = wait_bar(bar_full(pos), parity(pos)) && wait_bar(bar_pfull, i & 1);
+      ok = wait_bar(bar_full(pos), parity(pos));
+      if (ok && j == tiles_a - 1 && (n_a & 15)) {
+        // The rows behind p0 in the last granule of the local past may hold anything.  Their weight is 0, but 0 x NaN
+        // is NaN: they become zeros here, where the tile is waited for anyway.
+        uint4* granule = reinterpret_cast<uint4*>(base_generic + s * kTileBytes + ((n_a - j * kBN) >> 4) * 4096);
+        for (int v = lane; v < 256; v += 32)              // [group of 8 rows][channel half][row][vector]
+          if ((v >> 7) * 8 + ((v >> 3) & 7) >= (n_a & 15)) granule[v] = make_uint4(0, 0, 0, 0);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      }
+      ok = ok && wait_bar(bar_pfull, i & 1);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
@@ -658,8 +667,8 @@ int launch_attention_decode_t(const actqkv_config* cfg, const Batch& b, const At
   const cuuint64_t str[2] = {cuuint64_t(kD) * 2, cuuint64_t(Hq) * kD * 2};
   const cuuint32_t box[3] = {64, cuuint32_t(G), cuuint32_t(nt)};
   const uint64_t granules = uint64_t(b.n_layers) * cfg->n_phys_pages * Hkv * (cfg->page_tokens / 16);
-  if (!encode(&tm[0], a.q, 3, dims, str, box) || !encode_step_groups(&tm[1], a.k_win, uint64_t(U) * nt, Hkv) ||
-      !encode_step_groups(&tm[2], a.v_win, uint64_t(U) * nt, Hkv) || !encode_granules(&tm[3], a.k_pages, granules) ||
+  if (!encode(&tm[0], a.q, 3, dims, str, box) || !encode_unit_groups(&tm[1], a.k_win, U, nt, Hkv) ||
+      !encode_unit_groups(&tm[2], a.v_win, U, nt, Hkv) || !encode_granules(&tm[3], a.k_pages, granules) ||
       !encode_granules(&tm[4], a.v_pages, granules))
     return ACTQKV_ERR_LAUNCH;
   TcParams p;

@@ -545,6 +545,14 @@ inline bool encode_step_groups(CUtensorMap* tm, const void* base, uint64_t n_tok
   const cuuint32_t box[4] = {64, 8, 2, 1};
   return encode(tm, base, 4, dims, str, box);
 }
+// The same with the unit as a dimension of its own: a box that runs past the unit's last token brings zeros, not the
+// next unit's tokens.
+inline bool encode_unit_groups(CUtensorMap* tm, const void* base, int units, int n_tokens, int n_heads) {
+  const cuuint64_t dims[5] = {64, cuuint64_t(n_tokens), 2, cuuint64_t(n_heads), cuuint64_t(units)};
+  const cuuint64_t str[4] = {cuuint64_t(n_heads) * 256, 128, 256, cuuint64_t(n_tokens) * n_heads * 256};
+  const cuuint32_t box[5] = {64, 8, 2, 1, 1};
+  return encode(tm, base, 5, dims, str, box);
+}
 
 // Tensor map without swizzle for fp32 (fp32 = true) or bf16 data: the box lands in shared memory
 // densely, innermost dimension first.
