@@ -548,10 +548,11 @@ attention_decode_t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid
         if (key == r) store_lse(g0 + r, m[r], l[r]);
       }
     } else {
-      // the ranks' partial results meet: O over the ring, which no copy or product uses any more
+      // the ranks' partial results meet: O over the ring, which no copy or product uses any more -- unless a wait gave
+      // up: copies may then still be landing there, and the rank's empty result is its sum of 0 alone
 #pragma unroll
       for (int r = 0; r < RS; ++r) {
-        part[(g0 + r) * kD + key] = o[r];
+        if (have) part[(g0 + r) * kD + key] = o[r];
         if (key == r) { ml[g0 + r] = have ? m[r] : -INFINITY; ml[R + g0 + r] = l[r]; }
       }
       __syncwarp();
@@ -562,45 +563,46 @@ attention_decode_t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid
   if (n_ranks > 1) {
     if (warp >= W0) cluster_sync_all();      // the softmax warps' first one
     // every rank finishes an equal share of the (row, V channels) items
-          constexpr int V = R < 16 ? 1 : 4;                   // few rows: one channel each is a single round, with fewer registers
-          const int items = rows * (kD / V), chunk = (items + n_ranks - 1) / n_ranks, end = min(items, (rank + 1) * chunk);
-          for (int e = rank * chunk + tid; e < end; e += kThreads) {
-            const int r = e / (kD / V), ch = V * (e % (kD / V));
-            float pm[kMaxRanks], pl[kMaxRanks], po[kMaxRanks][V], mm = -INFINITY;
-    #pragma unroll
-            for (int k = 0; k < kMaxRanks; ++k)
-              if (k < n_ranks) {
-                pm[k] = ld_peer(smem_u32(ml + r), k);
-                pl[k] = ld_peer(smem_u32(ml + R + r), k);
-                if constexpr (V == 1) po[k][0] = ld_peer(smem_u32(part + r * kD + ch), k);
-                else ld_peer4(smem_u32(part + r * kD + ch), k, reinterpret_cast<float(&)[4]>(po[k]));
-              }
-    #pragma unroll
-            for (int k = 0; k < kMaxRanks; ++k)
-              if (k < n_ranks) mm = fmaxf(mm, pm[k]);
-            float ll = 0.f, oo[V] = {};
-    #pragma unroll
-            for (int k = 0; k < kMaxRanks; ++k)
-              if (k < n_ranks) {
-                const float w = pm[k] == -INFINITY ? 0.f : ex2(pm[k] - mm);
-                ll = fmaf(w, pl[k], ll);
-    #pragma unroll
-                for (int v = 0; v < V; ++v) oo[v] = fmaf(w, po[k][v], oo[v]);
-              }
-    #pragma unroll
-            for (int v = 0; v < V; ++v) oo[v] = ll > 0.f ? oo[v] / ll : 0.f;
-            const size_t at = row_out(r) + ch;
-            if constexpr (V == 1) {
-              if (p.out_bf16) static_cast<__nv_bfloat16*>(p.a.out)[at] = __float2bfloat16_rn(oo[0]);
-              else static_cast<float*>(p.a.out)[at] = oo[0];
-            } else if (p.out_bf16) {
-              *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(p.a.out) + at) =
-                  make_uint2(pack_bf16(oo[0], oo[1]), pack_bf16(oo[2], oo[3]));
-            } else {
-              *reinterpret_cast<float4*>(static_cast<float*>(p.a.out) + at) = make_float4(oo[0], oo[1], oo[2], oo[3]);
-            }
-            if (ch == 0) store_lse(r, mm, ll);
-          }
+    constexpr int V = R < 16 ? 1 : 4;                   // few rows: one channel each is a single round, with fewer registers
+    const int items = rows * (kD / V), chunk = (items + n_ranks - 1) / n_ranks, end = min(items, (rank + 1) * chunk);
+    for (int e = rank * chunk + tid; e < end; e += kThreads) {
+      const int r = e / (kD / V), ch = V * (e % (kD / V));
+      float pm[kMaxRanks], pl[kMaxRanks], po[kMaxRanks][V], mm = -INFINITY;
+#pragma unroll
+      for (int k = 0; k < kMaxRanks; ++k)
+        if (k < n_ranks) {
+          pm[k] = ld_peer(smem_u32(ml + r), k);
+          pl[k] = ld_peer(smem_u32(ml + R + r), k);
+          if constexpr (V == 1) po[k][0] = ld_peer(smem_u32(part + r * kD + ch), k);
+          else ld_peer4(smem_u32(part + r * kD + ch), k, reinterpret_cast<float(&)[4]>(po[k]));
+        }
+#pragma unroll
+      for (int k = 0; k < kMaxRanks; ++k)
+        if (k < n_ranks) mm = fmaxf(mm, pm[k]);
+      float ll = 0.f, oo[V] = {};
+#pragma unroll
+      for (int k = 0; k < kMaxRanks; ++k)
+        if (k < n_ranks) {
+          if (pl[k] == 0.f) continue;       // an empty partial result, whatever its O holds
+          const float w = ex2(pm[k] - mm);
+          ll = fmaf(w, pl[k], ll);
+#pragma unroll
+          for (int v = 0; v < V; ++v) oo[v] = fmaf(w, po[k][v], oo[v]);
+        }
+#pragma unroll
+      for (int v = 0; v < V; ++v) oo[v] = ll > 0.f ? oo[v] / ll : 0.f;
+      const size_t at = row_out(r) + ch;
+      if constexpr (V == 1) {
+        if (p.out_bf16) static_cast<__nv_bfloat16*>(p.a.out)[at] = __float2bfloat16_rn(oo[0]);
+        else static_cast<float*>(p.a.out)[at] = oo[0];
+      } else if (p.out_bf16) {
+        *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(p.a.out) + at) =
+            make_uint2(pack_bf16(oo[0], oo[1]), pack_bf16(oo[2], oo[3]));
+      } else {
+        *reinterpret_cast<float4*>(static_cast<float*>(p.a.out) + at) = make_float4(oo[0], oo[1], oo[2], oo[3]);
+      }
+      if (ch == 0) store_lse(r, mm, ll);
+    }
     cluster_sync_all();                     // a peer may still read this CTA's part
   }
 

@@ -56,3 +56,33 @@ def test_decode_wait_that_runs_out_sets_the_timeout_bit_and_the_context_stays_us
         again, s = run(cfg, splits, w)
         assert s == 0
         assert torch.equal(again, good1 if splits == 1 else good3)
+
+
+@pytest.mark.parametrize("nt,splits,dropped", [(1, 1, 0), (1, 4, 0), (1, 8, 1), (4, 4, 1), (8, 2, 2), (8, 8, 0)])
+def test_what_a_rank_that_gave_up_leaves_behind_does_not_reach_the_output(nt, splits, dropped):
+    """The ranks of a decode step merge on chip.  One whose wait ran out may have copies on their way into the memory its
+    partial result would take, so that result counts as empty: the output is finite, whatever else is wrong."""
+    import torch
+    from paper_2502_13542_b200 import binding as B
+    spec = wl.llama3_8b_layer().replace(context=4096, n_local_prev=2048, k_blocks=8, cap_blocks=8)
+    kw = dict(out_dtype=B.F32, max_context=4200)
+    cfg = B.make_config(spec, **kw)
+    st = B.RetrievalState(cfg)
+    gen = torch.Generator(device="cuda").manual_seed(9)
+
+    def rnd(n, h):
+        return torch.randn(1, n, h, 128, device="cuda", generator=gen).to(torch.bfloat16)
+
+    B.append_window(B.make_config(spec.replace(window=4096), **kw), st.batch, rnd(4096, 8), rnd(4096, 8), 4096, st.pos0, st.k_pages,
+                    st.v_pages, st.page_table, st.repr_k, st.repr_inv_norm, st.status)
+    st.set_positions([4096])
+    q, k, v = rnd(nt, 32), rnd(nt, 8), rnd(nt, 8)
+    ws = torch.empty(max(16, B.decode_workspace_bytes(cfg, st.batch, nt, splits)), dtype=torch.uint8, device="cuda")
+    cfg.test_wait_limit, cfg.test_drop_k_tile = 2000, dropped
+    for _ in range(3):
+        out = torch.full((1, nt, 32, 128), float("nan"), device="cuda")
+        B.decode_attention(cfg, st.batch, q, k, v, nt, st.k_pages, st.v_pages, st.page_table, st.pos0, st.sel_idx, st.sel_count,
+                           out, None, n_splits=splits, workspace=ws, status=st.status)
+        torch.cuda.synchronize()
+        assert int(st.status.item()) & B.DEV_TIMEOUT
+        assert torch.isfinite(out).all()
