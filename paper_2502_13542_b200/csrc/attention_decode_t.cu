@@ -268,7 +268,7 @@ attention_decode_t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid
   auto store_lse = [&](int r, float mm, float ll) {
     if (p.a.lse)
       p.a.lse[(size_t(unit) * p.n_q_heads + g * G + r % G) * nt + r / G] =
-          ll > 0.f ? (mm + log2f(ll)) * 0.6931471805599453f : -INFINITY;
+          ll == 0.f ? -INFINITY : (mm + log2f(ll)) * 0.6931471805599453f;
   };
   int issued = 0;                                         // tiles a producer has issued copies for
   if (warp == W0 || warp == W0 + 1) {
@@ -542,7 +542,7 @@ attention_decode_t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid
       for (int r = 0; r < RS; ++r) {
         if (r >= mine) break;
         const size_t at = row_out(g0 + r) + key;
-        const float v = l[r] > 0.f ? o[r] / l[r] : 0.f;
+        const float v = l[r] == 0.f ? 0.f : o[r] / l[r];      // (a sum that is not a number stays one)
         if (p.out_bf16) static_cast<__nv_bfloat16*>(p.a.out)[at] = __float2bfloat16_rn(v);
         else static_cast<float*>(p.a.out)[at] = v;
         if (key == r) store_lse(g0 + r, m[r], l[r]);
@@ -590,7 +590,7 @@ attention_decode_t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid
           for (int v = 0; v < V; ++v) oo[v] = fmaf(w, po[k][v], oo[v]);
         }
 #pragma unroll
-      for (int v = 0; v < V; ++v) oo[v] = ll > 0.f ? oo[v] / ll : 0.f;
+      for (int v = 0; v < V; ++v) oo[v] = ll == 0.f ? 0.f : oo[v] / ll;
       const size_t at = row_out(r) + ch;
       if constexpr (V == 1) {
         if (p.out_bf16) static_cast<__nv_bfloat16*>(p.a.out)[at] = __float2bfloat16_rn(oo[0]);
