@@ -526,8 +526,8 @@ bias_probe_ring_kernel(const __grid_constant__ CUtensorMap tm_q, BiasProbeParams
       run_count = p.stats_count[uh];
     }
     if (p.do_bias) {
-      // ---- pass 1, chunk by chunk as the rows land: sums of q and of (q - shift)^2, shift = row 0,
-      // on packed pairs of channels
+      // ---- pass 1, chunk by chunk as the rows land: sums of q - shift and of (q - shift)^2, shift = row 0,
+      // on packed pairs of channels (a channel without variance has both at exactly 0)
       uint64_t shift2[N2], s1p[N2], s2p[N2];
 #pragma unroll
       for (int e = 0; e < N2; ++e) { s1p[e] = 0; s2p[e] = 0; shift2[e] = 0; }
@@ -552,7 +552,7 @@ bias_probe_ring_kernel(const __grid_constant__ CUtensorMap tm_q, BiasProbeParams
 #pragma unroll
             for (int e = 0; e < N2; ++e) {
               const uint64_t d = tc::sub2(x[e], shift2[e]);
-              s1p[e] = tc::add2(s1p[e], x[e]);
+              s1p[e] = tc::add2(s1p[e], d);
               s2p[e] = tc::fma2(d, d, s2p[e]);
             }
           }
@@ -571,10 +571,9 @@ bias_probe_ring_kernel(const __grid_constant__ CUtensorMap tm_q, BiasProbeParams
       if (tid < D) {
         double n = double(W);
         const double sh0 = double(shift_s[tid]);
-        const double sq = double(sum_a[tid]), b2 = double(sum_b[tid]);
-        const double a = sq - n * sh0;             // sum (q - shift)
-        double mean = sq / n, m2 = fmax(b2 - a * a / n, 0.0);
-        qsum_s[tid] = sum_a[tid];
+        const double a = double(sum_a[tid]), b2 = double(sum_b[tid]);
+        double mean = sh0 + a / n, m2 = fmax(b2 - a * a / n, 0.0);
+        qsum_s[tid] = float(n * sh0 + a);
         if (running) {
           const double na = double(run_count), mean_a = double(run_mean), m2_a = double(run_m2);
           const double nn = na + n, delta = mean - mean_a, w = n / nn;
@@ -604,18 +603,18 @@ bias_probe_ring_kernel(const __grid_constant__ CUtensorMap tm_q, BiasProbeParams
     }
     float a_tot = 0.f;
     const bool four_rows = p.do_bias && p.do_probe && !p.phi_full && VPR >= 4;
-    // ||phi_j||_1 is summed as sum_c q (q iv - 2 mean iv) + sum_c mean^2 iv: two packed operations per
-    // pair of channels instead of three, on both paths alike (so every form of the call gives the same
-    // bits); the full phi, when asked for, is written as (q - mean)^2 iv.
-    uint64_t nb2[N2];
-    float phi_const = 0.f;                            // this thread's channels of sum_c mean^2 iv
+    // phi as (q - mean)^2 iv, in this order on both paths, so that every form of the call gives the same bits.  (The
+    // expanded sum_c q (q iv - 2 mean iv) + sum_c mean^2 iv is an operation shorter, but where |mean| is many sigma it
+    // cancels: an error of 1e-2 per channel at 300 sigma, and a channel without variance drowns all others.)
+    auto phi_sum = [&](const uint64_t (&x)[N2]) {
+      uint64_t sum = 0;
 #pragma unroll
-    for (int e = 0; e < N2; ++e) {
-      const uint64_t mi = tc::mul2(mc2[e], iv2[e]);
-      nb2[e] = tc::mul2(mi, tc::pack2(-2.f, -2.f));
-      const uint64_t mm = tc::mul2(mi, mc2[e]);
-      phi_const += tc::lo2(mm) + tc::hi2(mm);
-    }
+      for (int e = 0; e < N2; ++e) {
+        const uint64_t d = tc::sub2(x[e], mc2[e]);
+        sum = tc::fma2(tc::mul2(d, d), iv2[e], sum);
+      }
+      return tc::lo2(sum) + tc::hi2(sum);
+    };
     for (int c = 0; c < n_chunks; ++c, ++seq) {
       const uint32_t slot = seq % kRingSlots;
       wait_bar(bar_full + slot, (seq / kRingSlots) & 1);
@@ -633,10 +632,7 @@ bias_probe_ring_kernel(const __grid_constant__ CUtensorMap tm_q, BiasProbeParams
         for (int j = 0; j < 4; ++j) {
           const bool live = r_base + j * RL < W;
           Pairs<T>::get(live ? *reinterpret_cast<const uint4*>(src + size_t(j) * RL * D) : make_uint4(0, 0, 0, 0), x[j]);
-          uint64_t part2 = 0;
-#pragma unroll
-          for (int e = 0; e < N2; ++e) part2 = tc::fma2(x[j][e], tc::fma2(x[j][e], iv2[e], nb2[e]), part2);
-          part[j] = live ? fmaxf(tc::lo2(part2) + tc::hi2(part2) + phi_const, 0.f) : 0.f;
+          part[j] = live ? phi_sum(x[j]) : 0.f;
         }
         constexpr int H1 = VPR / 2, H2 = VPR / 4;
         const bool up1 = lane & H1, up2 = lane & H2;
@@ -666,7 +662,6 @@ bias_probe_ring_kernel(const __grid_constant__ CUtensorMap tm_q, BiasProbeParams
           Pairs<T>::get(live ? *reinterpret_cast<const uint4*>(src + size_t(k) * RL * D) : make_uint4(0, 0, 0, 0), x);
           float a;
           if (p.do_bias) {
-            uint64_t part2 = 0;
             if (p.phi_full && live) {
               float* dst = p.phi_full + (size_t(unit) * W + r) * row_stride + size_t(h) * D + cv * VN;
 #pragma unroll
@@ -676,9 +671,7 @@ bias_probe_ring_kernel(const __grid_constant__ CUtensorMap tm_q, BiasProbeParams
                 *reinterpret_cast<float2*>(dst + 2 * e) = make_float2(tc::lo2(ph), tc::hi2(ph));
               }
             }
-#pragma unroll
-            for (int e = 0; e < N2; ++e) part2 = tc::fma2(x[e], tc::fma2(x[e], iv2[e], nb2[e]), part2);   // as on the four-row path
-            float part = live ? fmaxf(tc::lo2(part2) + tc::hi2(part2) + phi_const, 0.f) : 0.f;
+            float part = live ? phi_sum(x) : 0.f;
 #pragma unroll
             for (int o = VPR >> 1; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
             a = part;                                // every lane of the row holds the same sum
