@@ -793,14 +793,18 @@ template <typename T, int D>
 int launch_d(const actqkv_config* cfg, const Batch& b, BiasProbeParams& p, cudaStream_t st) {
   const int W = p.n_tokens;
   const int cy = p.do_probe ? p.group : 1;
-  // Many items: the persistent streaming kernel (throughput); few: the cluster kernel (latency).
-  const int n_sm = kNumSMs;
-  // A cluster serves the cy heads of a KV group with 8 / cy CTAs per head, one CTA per SM: once that is more than
-  // one wave, items take fewer SMs and less time on the streaming kernel (8 prompts, 256 items of 512 rows:
-  // 46 us in 512 cluster CTAs, 17 us here).
-  const int cluster_split = std::max(1, 8 / cy);
-  if (b.units() * cfg->n_q_heads * cluster_split > n_sm) {
-    const int rc = launch_ring<T, D>(cfg, b, p, st, n_sm);
+  // Many items: the persistent streaming kernel (throughput); few: the cluster kernel (latency).  A cluster serves the
+  // cy heads of a KV group with `split` CTAs per head.  Tiles of up to 32 KiB in bf16 leave room for two CTAs per SM:
+  // those clusters are the faster ones as long as all of them are resident at once (bf16, D = 128, G = 4: 128 items of
+  // 256 rows 16.4 against 17.5 us, 160 items 24.5 against 19.5; G = 1, 32 items of 512 rows, bias alone 12.4 against
+  // 20.5, 64 items 20.5 both).  With one CTA per SM clusters of eight stop fitting side by side before the SMs are full
+  // (32 items of 512 rows 14.3 against 21.5, 64 items 23.5 against 21.5; fp32, D = 64: 10.2 against 13.3, 15.2 against
+  // 13.3): half the SMs are the line.
+  int split = std::max(1, kMaxCluster / cy);
+  while (split > 1 && (W + split - 1) / split < 32) split >>= 1;
+  const bool two_per_sm = sizeof(T) == 2 && size_t((W + split - 1) / split) * D * sizeof(T) <= 32 * 1024;
+  if (int64_t(b.units()) * cfg->n_q_heads * split > (two_per_sm ? 2 * kNumSMs : kNumSMs / 2)) {
+    const int rc = launch_ring<T, D>(cfg, b, p, st, kNumSMs);
     if (rc <= 0) return rc;
   }
   auto kern = bias_probe_kernel<T, D>;
@@ -808,40 +812,35 @@ int launch_d(const actqkv_config* cfg, const Batch& b, BiasProbeParams& p, cudaS
   constexpr int RL = kThreads / (D / VN), NP = kThreads / D;
   // Clusters stay within the portable size of 8: 16-CTA clusters were measured slower here (they
   // are scheduled one GPC at a time and their barrier costs more than the extra SMs bring).
-  for (int max_cluster = 8; max_cluster >= 8; max_cluster >>= 1) {
-    int split = max_cluster / cy;
-    if (split < 1) split = 1;
-    while (split > 1 && (W + split - 1) / split < 32) split >>= 1;
-    p.split = split;
-    p.rows_per_cta = (W + split - 1) / split;
-    p.box_rows = std::min(p.rows_per_cta, 256);                          // a box dimension holds at most 256
-    p.rows_alloc = (p.rows_per_cta + p.box_rows - 1) / p.box_rows * p.box_rows;
-    CUtensorMap tm_q;
-    if (!encode_q<T, D>(&tm_q, p, b.units(), p.box_rows)) return ACTQKV_ERR_LAUNCH;
-    const size_t tile_bytes = (size_t(p.rows_alloc) * D * sizeof(T) + 127) & ~size_t(127);
-    const size_t smem = tile_bytes + sizeof(float) * (size_t(2) * RL * D + 2 * NP * D + 6 * D + 4 + 32 +
-                                                       ((p.rows_per_cta + 3) & ~3) + 2 * kMaxCluster +
-                                                       4 * kMaxCluster * D) + 16;
-    if (smem > 220 * 1024) return ACTQKV_ERR_SHAPE;
-    static std::atomic<bool> opted_in[kMaxDevices], carved[kMaxDevices];
-    if (!opt_in_shared_memory(kern, 220 * 1024, opted_in)) return ACTQKV_ERR_LAUNCH;
-    prefer_max_shared(kern, carved);
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(split, cfg->n_q_heads, b.units());
-    lc.blockDim = dim3(kThreads, 1, 1);
-    lc.dynamicSmemBytes = smem;
-    lc.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = split;
-    attr[0].val.clusterDim.y = cy;
-    attr[0].val.clusterDim.z = 1;
-    allow_early_launch(attr[1]);
-    lc.attrs = attr;
-    lc.numAttrs = 2;
-    if (cudaLaunchKernelEx(&lc, kern, tm_q, p) == cudaSuccess) return launch_status();
-    (void)cudaGetLastError();
-  }
+  p.split = split;
+  p.rows_per_cta = (W + split - 1) / split;
+  p.box_rows = std::min(p.rows_per_cta, 256);                          // a box dimension holds at most 256
+  p.rows_alloc = (p.rows_per_cta + p.box_rows - 1) / p.box_rows * p.box_rows;
+  CUtensorMap tm_q;
+  if (!encode_q<T, D>(&tm_q, p, b.units(), p.box_rows)) return ACTQKV_ERR_LAUNCH;
+  const size_t tile_bytes = (size_t(p.rows_alloc) * D * sizeof(T) + 127) & ~size_t(127);
+  const size_t smem = tile_bytes + sizeof(float) * (size_t(2) * RL * D + 2 * NP * D + 6 * D + 4 + 32 +
+                                                     ((p.rows_per_cta + 3) & ~3) + 2 * kMaxCluster +
+                                                     4 * kMaxCluster * D) + 16;
+  if (smem > 220 * 1024) return ACTQKV_ERR_SHAPE;
+  static std::atomic<bool> opted_in[kMaxDevices], carved[kMaxDevices];
+  if (!opt_in_shared_memory(kern, 220 * 1024, opted_in)) return ACTQKV_ERR_LAUNCH;
+  prefer_max_shared(kern, carved);
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(split, cfg->n_q_heads, b.units());
+  lc.blockDim = dim3(kThreads, 1, 1);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = split;
+  attr[0].val.clusterDim.y = cy;
+  attr[0].val.clusterDim.z = 1;
+  allow_early_launch(attr[1]);
+  lc.attrs = attr;
+  lc.numAttrs = 2;
+  if (cudaLaunchKernelEx(&lc, kern, tm_q, p) == cudaSuccess) return launch_status();
+  (void)cudaGetLastError();
   return ACTQKV_ERR_LAUNCH;
 }
 
