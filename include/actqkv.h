@@ -165,7 +165,8 @@ int32_t actqkv_n_candidates(const actqkv_config* cfg, int64_t p0);
 
 /* The positions of the next step: writes pos0[i] = positions[i] and the matching candidate count
  * n_cand[i] (actqkv_n_candidates) for n_seq sequences.  `positions` is a HOST array, read before the call
- * returns; the values travel as kernel arguments, so nothing is copied and nothing waits.
+ * returns; the values travel as kernel arguments, so nothing is copied and nothing waits.  A stream that is being
+ * captured is refused (ACTQKV_ERR_UNSUPPORTED): every replay of the graph would set the same positions.
  *   pos0 [n_seq] int64 out;  n_cand [n_seq] int32 out, may be NULL.
  * Like actqkv_append_window it runs strictly after its predecessor and before its successor in the stream. */
 int actqkv_set_positions(const actqkv_config* cfg, int32_t n_seq, const int64_t* positions, int64_t* pos0,
@@ -341,8 +342,9 @@ int actqkv_append_window(const actqkv_config* cfg, const actqkv_batch* batch, co
  * Enqueues, in this order and with the same results, actqkv_bias_probe (when update_probe is non-zero),
  * actqkv_score_select, actqkv_retrieval_attention, actqkv_append_window and, when next_positions (HOST array of
  * n_next sequences) is given, actqkv_set_positions.  The struct holds the arguments of those calls under their
- * names; what may be NULL there may be NULL here.  n_next must be the batch's number of sequences (ACTQKV_ERR_SHAPE, nothing
- * is enqueued).  Returns the first error of a stage; the stages before it are enqueued. */
+ * names; what may be NULL there may be NULL here.  With next_positions, n_next must be the batch's number of sequences
+ * (ACTQKV_ERR_SHAPE) and the stream must not be capturing (ACTQKV_ERR_UNSUPPORTED); nothing is enqueued then.  Returns the
+ * first error of a stage; the stages before it are enqueued. */
 typedef struct actqkv_step_buffers {
   const void *q, *k_win, *v_win;
   void* out;

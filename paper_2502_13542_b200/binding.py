@@ -345,7 +345,9 @@ class RetrievalState:
 
         overlap_append: enqueue the append on a second stream, concurrent with the other stages (it
         reads only the step's own K / V and writes pages and table rows that no other stage of the
-        same step reads); the streams are joined before the step returns."""
+        same step reads); the streams are joined before the step returns.
+        A step that is being captured into a graph takes advance=False: the positions of a replay are set
+        ahead of it."""
         cfg, b = self.cfg, self.batch
         nt = n_tokens if n_tokens is not None else q.shape[-3]
         if fused and not overlap_append:      # one call into the library: enqueueing is what bounds small steps
@@ -357,6 +359,8 @@ class RetrievalState:
             if advance:
                 self.host_pos0 = after
             return
+        if advance and torch.cuda.is_current_stream_capturing():
+            raise ActQKVError("a captured step cannot advance: every replay would set the same positions")
 
         def fork_append():
             self._fork.record(main)

@@ -107,3 +107,33 @@ def test_positions_of_a_state():
         st.step(x, x[:, :, :2].contiguous(), x[:, :, :2].contiguous(), torch.zeros_like(x))
     torch.cuda.synchronize()
     assert pool.tolist() == [400] * 3 + [-5] * 5 and int(st.stats_count.sum()) == 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kw", [{}, {"fused": False}, {"overlap_append": True}])
+def test_a_capture_takes_no_positions(kw):
+    """Their values would be frozen into the graph: refused, with nothing of the step enqueued and the capture and
+    the state as they were."""
+    import torch
+    from paper_2502_13542_b200 import binding as B
+    spec = wl.tiny_pr1()
+    st = B.RetrievalState(B.make_config(spec))
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    q, k, v = (torch.randn(1, spec.window, h, 64, device="cuda", generator=gen) for h in (4, 2, 2))
+    out = torch.zeros_like(q)
+    st.set_positions([640])
+    st.step(q, k, v, out, advance=False, **kw)
+    torch.cuda.synchronize()
+    seen = st.stats_count.clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        with pytest.raises(B.ActQKVError):
+            st.set_positions([0])
+        with pytest.raises(B.ActQKVError):
+            st.step(q, k, v, out, **kw)
+        st.step(q, k, v, out, advance=False, **kw)
+    assert st.host_pos0 == [640]
+    graph.replay()
+    torch.cuda.synchronize()
+    assert st.pos0.tolist() == [640] and torch.equal(st.stats_count, seen + spec.window)
+    assert int(st.status.item()) == 0
