@@ -256,9 +256,11 @@ int actqkv_score_select(const actqkv_config* cfg, const actqkv_batch* batch, con
  *   lse          [U][Hq][n_tokens]      fp32 out, may be NULL (natural-log sum of exp)
  * bf16, D = 128, pages of 16 to 128 tokens run on tcgen05 kernels: steps of at most 32 rows (n_tokens * G) on the
  * transposed decode kernel; batches of 33 to 128 rows per KV head and 16-token pages that fill the SMs on the
- * padded decode kernel (see actqkv_decode_attention for its split form); every other step, a multiple of a tile or not, on a prefill kernel
- * (CTA pairs where they fill the SMs in one wave, else two query tiles per CTA with the key stream cut over a
- * cluster).  Every other type or head size runs on the general fp32-accumulate kernel.
+ * padded decode kernel (see actqkv_decode_attention for its split form); every other step, a multiple of a tile or not,
+ * on a prefill kernel (CTA pairs where they fill the SMs in one wave, else two query tiles per CTA with the key stream
+ * cut over a cluster).  Every other type or head size runs on the general fp32-accumulate kernel, and so do fp32 results
+ * (out_dtype) of steps that are neither whole 128-token tiles (16-token pages, or an even G) nor at most 128 rows (16-token
+ * pages, 128 a multiple of G): there the weights are held in fp32.
  * Preconditions of the tcgen05 kernels (the general kernel has none of them):
  *  - Steps of whole 128-token tiles with an even G, and steps of 33 to 128 rows: p0 need not sit on a page boundary, but
  *    the rows of the last, partly filled cache page that lie past p0 must hold finite values: they are masked out of
