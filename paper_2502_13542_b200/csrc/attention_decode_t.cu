@@ -549,10 +549,10 @@ attention_decode_t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid
       }
     } else {
       // the ranks' partial results meet: O over the ring, which no copy or product uses any more -- unless a wait gave
-      // up: copies may then still be landing there, and the rank's empty result is its sum of 0 alone
+      // up: copies may then still be landing there, and the merge reads from the rank's sum of 0 that there is nothing
 #pragma unroll
       for (int r = 0; r < RS; ++r) {
-        if (have) part[(g0 + r) * kD + key] = o[r];
+        part[(g0 + r) * kD + key] = o[r];
         if (key == r) { ml[g0 + r] = have ? m[r] : -INFINITY; ml[R + g0 + r] = l[r]; }
       }
       __syncwarp();
