@@ -20,7 +20,7 @@ def test_nan_stays_nan(hq, hkv, units, nt, page):
     spec = wl.llama3_8b_layer().replace(n_q_heads=hq, n_kv_heads=hkv, page_tokens=page, k_blocks=2, cap_blocks=2,
                                         context=past + nt, n_local_prev=256)
     per_seq = -(-(past + nt) // page) + 1
-    kw = dict(n_phys_pages=units * per_seq, max_pages=per_seq, out_dtype=B.F32)
+    kw = dict(n_phys_pages=units * per_seq, max_pages=per_seq)
     cfg = B.make_config(spec, **kw)
     st = B.RetrievalState(cfg, n_seq=units, page_table=torch.arange(units * per_seq, dtype=torch.int32).reshape(units, per_seq))
     gen = torch.Generator(device="cuda").manual_seed(nt)
@@ -37,7 +37,7 @@ def test_nan_stays_nan(hq, hkv, units, nt, page):
     q, k, v = rnd(nt, hq), rnd(nt, hkv), rnd(nt, hkv)
 
     def rows_with_nan():
-        out = torch.zeros(units, nt, hq, 128, device="cuda")
+        out = torch.zeros(units, nt, hq, 128, device="cuda", dtype=torch.bfloat16)
         lse = torch.zeros(units, hq, nt, device="cuda")
         B.retrieval_attention(cfg, st.batch, q, k, v, nt, st.k_pages, st.v_pages, st.page_table, st.pos0, st.sel_idx,
                               st.sel_count, out, lse, st.status)
