@@ -526,8 +526,8 @@ bias_probe_ring_kernel(const __grid_constant__ CUtensorMap tm_q, BiasProbeParams
       run_count = p.stats_count[uh];
     }
     if (p.do_bias) {
-      // ---- pass 1, chunk by chunk as the rows land: sums of q - shift and of (q - shift)^2, shift = row 0,
-      // on packed pairs of channels (a channel without variance has both at exactly 0)
+      // ---- pass 1, chunk by chunk as the rows land: sums of q and of (q - shift)^2, shift = row 0,
+      // on packed pairs of channels
       uint64_t shift2[N2], s1p[N2], s2p[N2];
 #pragma unroll
       for (int e = 0; e < N2; ++e) { s1p[e] = 0; s2p[e] = 0; shift2[e] = 0; }
@@ -552,7 +552,7 @@ bias_probe_ring_kernel(const __grid_constant__ CUtensorMap tm_q, BiasProbeParams
 #pragma unroll
             for (int e = 0; e < N2; ++e) {
               const uint64_t d = tc::sub2(x[e], shift2[e]);
-              s1p[e] = tc::add2(s1p[e], d);
+              s1p[e] = tc::add2(s1p[e], x[e]);
               s2p[e] = tc::fma2(d, d, s2p[e]);
             }
           }
@@ -571,9 +571,10 @@ bias_probe_ring_kernel(const __grid_constant__ CUtensorMap tm_q, BiasProbeParams
       if (tid < D) {
         double n = double(W);
         const double sh0 = double(shift_s[tid]);
-        const double a = double(sum_a[tid]), b2 = double(sum_b[tid]);
-        double mean = sh0 + a / n, m2 = fmax(b2 - a * a / n, 0.0);
-        qsum_s[tid] = float(n * sh0 + a);
+        const double sq = double(sum_a[tid]), b2 = double(sum_b[tid]);
+        const double a = sq - n * sh0;             // sum (q - shift)
+        double mean = sq / n, m2 = fmax(b2 - a * a / n, 0.0);
+        qsum_s[tid] = sum_a[tid];
         if (running) {
           const double na = double(run_count), mean_a = double(run_mean), m2_a = double(run_m2);
           const double nn = na + n, delta = mean - mean_a, w = n / nn;
