@@ -267,7 +267,7 @@ int actqkv_score_select(const actqkv_config* cfg, const actqkv_batch* batch, con
  *    the softmax yet may still enter the P V product with weight 0, and 0 x NaN is NaN.  A zero-initialised pool
  *    satisfies this, and actqkv_append_window zero-fills the rest of the last page it touches.
  *  - Steps of whole 128-token tiles with an even G multiply P and V in fp16: |v| <= 65504 (larger finite values
- *    saturate); the others take P as two bf16 terms. */
+ *    saturate); the others take P as two bf16 terms, of up to 2^32, and sum in fp32: |v| <= 2^96 / (number of keys). */
 int actqkv_retrieval_attention(const actqkv_config* cfg, const actqkv_batch* batch, const void* q,
                                const void* k_win, const void* v_win, int32_t n_tokens,
                                const void* k_pages, const void* v_pages, const int32_t* page_table,

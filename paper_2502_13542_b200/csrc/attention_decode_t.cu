@@ -24,7 +24,7 @@
 // each: K producer (and Q), V producer, issuer of Q K^T, issuer of P V (one issuer for both holds the next Q K^T back
 // behind the wait for P; with it and a merge of one row per round: 158.9 us for six layers of one sequence, 152.9
 // without).  K and V tiles share one ring of 32 KiB slots, K0 V0 K1 V1 ...; a tile is eight boxes of one 16-token
-// granule.  The running maximum moves only when a score exceeds it by 2^64 (P has fp32's range), which is a vote per
+// granule.  The running maximum moves only when a score exceeds it by 2^32 (P has fp32's range), which is a vote per
 // tile; the reduction over the 128 threads that a new maximum takes is the rare path.
 // Measured against the padded form, whole decode steps as graphs: 64 sequences of 2k-8k tokens 528 -> 390 us for
 // two layers (the K / V stream alone 385 us at the measured copy bandwidth), 16 of 32k-131k 202 -> 166 us, one
@@ -46,8 +46,9 @@ constexpr int kMaxRanks = 8;
 constexpr int kMaxRows = 32;
 constexpr uint32_t kTileBytes = 32 * 1024;               // one K or V tile
 
-// P may reach 2^64 before the running maximum has to move: the sums of P and of P V stay below 2^90.
-constexpr float kMaxLag = 64.0f;
+// P may reach 2^32 before the running maximum has to move, as in the padded kernel: what it may reach is taken from the
+// range of V (six layers of one sequence 151.0 us with 2^64, 151.4 with this, 152.2 with 2^15, 153.9 with 2^8).
+constexpr float kMaxLag = kRescaleThreshold;
 
 // R: rows rounded up to 4, 8, 16 or 32; N: columns of S^T (a multiple of 16).  kDeep: one CTA per SM with six
 // ring slots, for grids that leave the SMs to one CTA each (and for 32 rows); else two CTAs of three.
@@ -685,7 +686,7 @@ int launch_attention_decode_t(const actqkv_config* cfg, const Batch& b, const At
   dp.spin_limit = cfg->test_wait_limit > 0 ? uint32_t(cfg->test_wait_limit) : 1u << 20;
   dp.drop_k_tile = cfg->test_wait_limit > 0 ? cfg->test_drop_k_tile : -1;
   // Ranks: doubled while every CTA has an SM to itself; one more doubling where two CTAs share an SM only then
-  // (128 to 148 streams), so that no SM is left idle beside a busy one.
+  // (75 to 148 streams), so that no SM is left idle beside a busy one.
   const int64_t pairs = int64_t(U) * Hkv;
   if (n_ranks <= 0) {
     n_ranks = 1;
