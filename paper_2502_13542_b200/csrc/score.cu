@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, 2) score_stream_kernel(Stre
   const int sub = lane / LPR, lir = lane - sub * LPR;
   const int per_seq = p.n_layers * p.n_kv_heads;
   auto smem = [](const void* x) { return uint32_t(__cvta_generic_to_shared(x)); };
-  auto candidates = [&](int seq) { return min(p.n_cand[seq], p.n_cap); };
+  auto candidates = [&](int seq) { return max(0, min(p.n_cand[seq], p.n_cap)); };      // the sums of groups only grow
 
   grid_launch_dependents();
   if (warp == 0) {                                  // running sum of the sequences' groups
