@@ -685,12 +685,13 @@ int launch_attention_decode_t(const actqkv_config* cfg, const Batch& b, const At
   DecodeTParams dp;
   dp.spin_limit = cfg->test_wait_limit > 0 ? uint32_t(cfg->test_wait_limit) : 1u << 20;
   dp.drop_k_tile = cfg->test_wait_limit > 0 ? cfg->test_drop_k_tile : -1;
-  // Ranks: doubled while every CTA has an SM to itself; one more doubling where two CTAs share an SM only then
+  // Ranks: doubled while all clusters are resident with an SM to each CTA (two sequences of 8 KV heads, 2,500 / 30,000
+  // tokens: 22.5 / 28.6 us over 8 CTAs each, which are two waves, 15.0 / 20.4 us over 4); one more doubling where two CTAs share an SM only then
   // (75 to 148 streams), so that no SM is left idle beside a busy one.
   const int64_t pairs = int64_t(U) * Hkv;
   if (n_ranks <= 0) {
     n_ranks = 1;
-    while (n_ranks < kMaxRanks && pairs * n_ranks * 2 <= kNumSMs) n_ranks *= 2;
+    while (n_ranks < kMaxRanks && pairs <= resident_clusters(n_ranks * 2)) n_ranks *= 2;
     if (rows <= 16 && n_ranks == 1 && pairs <= kNumSMs) n_ranks = 2;
   }
   dp.n_ranks = std::min(n_ranks, kMaxRanks);

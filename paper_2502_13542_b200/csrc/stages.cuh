@@ -101,6 +101,10 @@ int64_t attention_prefill_ctas(const actqkv_config* cfg, const Batch& b, int n_t
 bool attention_prefill_cuts(const actqkv_config* cfg, const Batch& b, int n_tokens);      // a key stream goes to several CTAs
 int launch_attention_prefill(const actqkv_config* cfg, const Batch& b, const AttnArgs& a, bool split_p, cudaStream_t st);
 
+// Clusters of `size` CTAs (2, 4 or 8) that are resident at once when every CTA takes an SM to itself.  A cluster lies
+// within one GPC, so it is fewer than the SMs would hold: 74, 33 and 15 on a B200.  Asked of the runtime once per device.
+int resident_clusters(int size);
+
 // Short steps of at most 32 rows (n_tokens * G): transposed products, the key stream cut over n_ranks CTAs of a
 // cluster (0: as many as fill the SMs), no workspace.
 bool attention_decode_t_supported(const actqkv_config* cfg, int n_tokens);
