@@ -37,7 +37,7 @@
  *    kernels of steps 1-5 let the next kernel of the stream start at once, and a
  *    kernel of this library that starts early reads, before it has waited for
  *    its predecessor, only buffers that steps 1-5 never write: the step's Q / K /
- *    V, pos0, page_table, the cache pages and table rows of tokens before pos0.
+ *    V, pos0, n_cand, page_table, the cache pages and table rows of tokens before pos0.
  *    It waits for its predecessor before it reads anything else and before it
  *    writes.  actqkv_append_window, which writes those buffers, writes only
  *    after its predecessor has ended and ends before its successor starts, and so does
@@ -141,7 +141,7 @@ typedef struct actqkv_config {
   int32_t probe_mode;    /* ACTQKV_PROBE_*: token weights of the probe-query                 */
   int32_t attention_kernel; /* ACTQKV_ATTN_*: 0 = pick by shape                              */
   /* Test hooks of the failure-detection path (leave both 0).  With test_wait_limit > 0 the decode
-   * attention kernel gives its device-side waits that many polls instead of the normal 2^24 and
+   * attention kernel gives its device-side waits that many polls instead of its normal limit and
    * never issues the K copy of tile test_drop_k_tile of each CTA, so that the wait for that tile runs
    * out: the kernel must set ACTQKV_DEV_TIMEOUT, return, and leave the context usable. */
   int32_t test_wait_limit;
@@ -276,13 +276,17 @@ int actqkv_retrieval_attention(const actqkv_config* cfg, const actqkv_batch* bat
 
 /* ---- step 5 for short steps (decode, Eq. 3) with the key stream split over several CTAs --------
  * The same attention as actqkv_retrieval_attention for steps of n_tokens <= 128 / G tokens
- * (G = Hq / Hkv; bf16, D = 128, 16-token pages), which packs the G query heads of a KV head into
- * one tensor-core tile so that K and V are read once per group.  With few (sequence, layer) units a
- * single CTA per KV head cannot fill the GPU: n_splits > 1 cuts every key stream into n_splits
- * shares; each share writes a partial result to `workspace` and a second kernel merges them
- * (n_splits = 0 picks the count that fills the SMs once; actqkv_decode_splits returns it).
- * Steps of at most 32 rows (n_tokens * G) cut the stream over up to 8 CTAs that merge on chip: the
- * workspace is then asked for as before but not used, and larger counts are taken as 8.
+ * (G = Hq / Hkv; bf16, D = 128, 16-token pages, G a divisor of 128; other pages and groups are served by
+ * actqkv_retrieval_attention only), which packs the G query heads of a KV head into one tensor-core tile so
+ * that K and V are read once per group.  With few (sequence, layer) units a single CTA per KV head cannot
+ * fill the GPU: n_splits > 1 cuts every key stream into n_splits shares.
+ *  - More than 32 rows (n_tokens * G): each share writes a partial result to `workspace` and a second
+ *    kernel merges them; n_splits = 0 takes the count that actqkv_decode_splits returns, which fills the
+ *    SMs once.
+ *  - At most 32 rows: the shares are the CTAs of a cluster, up to 8 (larger counts are taken as 8), and
+ *    merge on chip; n_splits = 0 takes as many as are resident at once, whatever actqkv_decode_splits
+ *    returns.  The workspace is not used, but the same one is asked for, so that the contract of a call does not
+ *    depend on which kernel serves it.
  *   workspace  device scratch of at least actqkv_decode_workspace_bytes(...) bytes, 16-byte
  *              aligned, caller-owned, contents undefined on entry and exit; may be NULL when
  *              the split count is 1.  Calls that overlap on the GPU need distinct workspaces.

@@ -80,7 +80,7 @@ inline void prefer_max_shared(Kernel kern, std::atomic<bool> (&done)[kMaxDevices
 // predecessor ends; since every link waits for its predecessor before it writes, the wait of the
 // last link still orders it after all of them.  What a kernel does BEFORE its wait may therefore
 // overlap any earlier kernel of the chain: it may read only what none of them writes (the step's
-// Q / K / V, positions, the page table, cache pages and table rows of past tokens).  The
+// Q / K / V, positions and candidate counts, the page table, cache pages and table rows of past tokens).  The
 // attention lets its successor start, too.  Kernels that write those (the append, set_positions) may start
 // early, but they wait before they write and do not let their successor start before they end.
 // Without the attribute the wait is a no-op.
