@@ -398,7 +398,7 @@ bool encode_q(CUtensorMap* tm, const BiasProbeParams& p, int units, int box_rows
 // The kernel is bound by its instruction pipes, not by memory or latency: a form that kept one whole
 // item per SM in shared memory (16 warps, phases in series) took the same 57 us for 32 layers,
 // three CTAs per SM are slower, and the packed fp32 and integer pipes both run at one warp
-// instruction per two cycles, which the unpacking of bf16 pairs and the 24 packed operations per
+// instruction per two cycles, which the unpacking of bf16 pairs and the 28 packed operations per
 // 16-byte vector fill.
 constexpr int kRingThreads = 256;           // consumer threads; warp 8 is the producer
 constexpr int kRingSlots = 4;
