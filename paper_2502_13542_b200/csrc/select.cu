@@ -13,19 +13,14 @@
 // sequence form a thread-block cluster, each takes its head's density, they exchange the values
 // through distributed shared memory, every CTA evaluates Eq. 12 for itself and the first one
 // writes the budget state back.
-#include <cooperative_groups.h>
-
 #include "common.cuh"
 #include "stages.cuh"
-
-namespace cg = cooperative_groups;
 
 using namespace actqkv;
 
 namespace {
 
 constexpr int kChainThreads = 1024;
-constexpr int kSelThreads = 256;
 
 struct ChainParams {
   const float* scores;
@@ -161,8 +156,13 @@ __device__ __forceinline__ uint32_t score_key(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// Exclusive scan of one int per thread over the CTA; returns the prefix, total in *total.
-__device__ __forceinline__ int block_exclusive_scan(int v, int* warp_tot, int* total) {
+// The threads of select_kernel that hold keys (the control warp behind them takes no part).
+template <int kKeys>
+__device__ __forceinline__ void key_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kKeys) : "memory"); }
+
+// Exclusive scan of one int per key thread; returns the prefix.
+template <int kKeys>
+__device__ __forceinline__ int key_exclusive_scan(int v, int* warp_tot) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int inc = v;
 #pragma unroll
@@ -170,39 +170,36 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_tot, int* t
     const int t = __shfl_up_sync(0xffffffffu, inc, o);
     if (lane >= o) inc += t;
   }
-  __syncthreads();
+  key_sync<kKeys>();
   if (lane == 31) warp_tot[warp] = inc;
-  __syncthreads();
-  int base = 0, tot = 0;
-  for (int w = 0; w < kSelThreads / 32; ++w) {
-    const int t = warp_tot[w];
-    if (w < warp) base += t;
-    tot += t;
-  }
-  *total = tot;
-  return base + inc - v;
+  key_sync<kKeys>();
+  const int before = __reduce_add_sync(0xffffffffu, lane < warp ? warp_tot[lane] : 0);
+  return before + inc - v;
 }
 
-// The largest threshold thr that at least c of the keys reach (0 < c < their number), three bits per step: warp w
-// counts the keys of at least thr | w << shift (w = 1..7), all of them, the first 256 from registers.  Done
+// The largest threshold thr that at least c of the keys reach (0 < c < their number), three or four bits per step: warp
+// w counts the keys of at least thr | w << shift (w >= 1), all of them, the first 256 from registers.  Done
 // early when exactly c keys reach thr.  Returns thr; at: the number of keys that reach it.  keys: padded with
 // zeros to 4 * n4, n4 a multiple of 32; tot: one count per warp, two sets used in turn.
-__device__ __forceinline__ uint32_t search_cth(int c, const uint32_t* keys, int n4, int (*tot)[kSelThreads / 32], int& at) {
+template <int kKeys>
+__device__ __forceinline__ uint32_t search_cth(int c, const uint32_t* keys, int n4, int (*tot)[kKeys / 32], int& at) {
+  constexpr int kWarps = kKeys / 32, kBits = kWarps == 16 ? 4 : 3;
+  static_assert(kWarps == 1 << kBits, "a threshold per warp");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint4* k4 = reinterpret_cast<const uint4*>(keys) + lane;
   const uint4 zero = make_uint4(0u, 0u, 0u, 0u), a = k4[0], b = n4 > 32 ? k4[32] : zero;
   uint32_t thr = 0u;
   int turn = 0;
-  for (int shift = 29;; shift -= 3) {
-    const int sh = max(shift, 0), top = shift < 0 ? 3 : 7;            // the last step has two bits
+  for (int shift = 32 - kBits;; shift -= kBits) {
+    const int sh = max(shift, 0), top = (1 << (kBits + min(shift, 0))) - 1;      // the last step may have fewer bits
     const uint32_t t = thr | (uint32_t(warp) << sh);
     auto reach = [&](const uint4& x) { return (int(x.x >= t) + int(x.y >= t)) + (int(x.z >= t) + int(x.w >= t)); };
     int cnt = reach(a) + reach(b);
     for (int i = 64; i < n4; i += 32) cnt += reach(k4[i]);
     cnt = __reduce_add_sync(0xffffffffu, cnt);
     if (lane == 0) tot[turn][warp] = cnt;
-    __syncthreads();
-    const int mine = tot[turn][lane & 7];                              // counts fall with w
+    key_sync<kKeys>();
+    const int mine = tot[turn][lane & (kWarps - 1)];                   // counts fall with w
     const int w = __popc(__ballot_sync(0xffffffffu, lane >= 1 && lane <= top && mine >= c));
     const int reached = __shfl_sync(0xffffffffu, mine, w);
     if (w > 0) { thr |= uint32_t(w) << sh; at = reached; }
@@ -211,117 +208,178 @@ __device__ __forceinline__ uint32_t search_cth(int c, const uint32_t* keys, int 
   }
 }
 
+// How many of the n keys (padded with zeros to a multiple of 4) come before key k of index i: larger ones, and equal
+// ones of a lower index.  The keys of the warps before and behind the own one need one comparison each.
+__device__ __forceinline__ int rank_of(uint32_t k, int i, const uint32_t* keys, int n) {
+  const uint4* k4 = reinterpret_cast<const uint4*>(keys);
+  const int own = (i & ~31) >> 2, end = (n + 3) >> 2;
+  int r = 0;
+#pragma unroll 4
+  for (int j = 0; j < own; ++j) {
+    const uint4 x = k4[j];
+    r += (int(x.x >= k) + int(x.y >= k)) + (int(x.z >= k) + int(x.w >= k));
+  }
+#pragma unroll 4
+  for (int j = own; j < end; ++j) {
+    const uint4 x = k4[j];
+    r += (int(x.x > k) + int(x.y > k)) + (int(x.z > k) + int(x.w > k));
+  }
+  const uint32_t same = __match_any_sync(0xffffffffu, k);              // equal keys inside the warp
+  return r + __popc(same & ((1u << (i & 31)) - 1u));
+}
+
 // kFused: the call holds one layer; the grid is launched as clusters of n_kv_heads CTAs (one
 // sequence each) and the cut-off chain of that layer is evaluated here (ch), else sel_count is
 // an input written by cutoff_chain_kernel.
 //
-// The kernel is a chain of short phases that run once per launch, and what bounds it is the first fetch of
-// their instructions: after the dependency wait it took 13.4k clk at 251 candidates and 17.4k at 307, of which
-// the density 3.3k-4.7k and the selection 4.6k-8.8k.  It sits idle until the scores exist, so it goes through all
-// phases once before the wait, on 32 made-up scores and without a global access (the rehearsal), and again
-// after it.  The c-th largest key is found by a search on its bits, three per step (each warp counts for a
-// threshold of its own), which ends as soon as a threshold separates exactly c keys; ranking every candidate
-// (n <= 256) and 8-bit radix passes (more) cost 4.6k and 7.5k clk, the search 1.9k and 2.9k.  After the wait:
-// 7.6k clk at 251 candidates, 10.1k at 307; a 32k window as a graph 268 -> 260 us for four layers.
-template <bool kFused>
-__global__ void __launch_bounds__(kSelThreads)
+// A chain of short phases on the critical path of a step, once per launch.  kKeys threads hold the keys, one warp
+// behind them (control) the chain: the key warps fetch the scores and leave one (maximum, Z, sum e x) per warp; control
+// merges these into the head's density, hands it to the cluster's CTAs by asynchronous remote stores that complete on
+// their barriers, adds up theirs and grants the count in fp64.  Meanwhile the key warps rank their keys against all
+// others, which needs no count; with the count a key is taken if its rank is below it, and one scan over the warps'
+// ballots places it.  Beyond kRankMax candidates the n^2 comparisons are longer than the chain beside them, and the
+// c-th largest key is found instead by a search on its bits (a threshold per warp and step), which ends as soon as a
+// threshold separates exactly c keys.  Score and selection of one layer, 60 of these pairs chained in a graph, us per pair
+// at 128 / 251 / 313 / 384 / 450 / 512 candidates: ranks 4.6 / 5.6 / 6.2 / 7.0 / 8.2 / 8.7, search 5.9 / 6.0 / 6.6 / 6.8 / 6.9 /
+// 6.6; with four sequences ranks 5.3 / 6.8 / 9.2 / 10.5 / 15.6 / 18.0, search 6.4 / 9.0 / 11.1 / 11.7 / 13.6 / 14.5.  With one thread
+// taking the density, a cluster barrier and a three-bit search after the count: 6.9 / 7.5 / 8.0 / 8.2 / 8.4 / 8.3 and 7.5 /
+// 9.5 / 12.9 / 13.7 / 14.9 / 15.2.
+// What is left is bound by the first fetch of the instructions, so the kernel goes through all
+// phases once before the dependency wait, on 32 made-up scores and without a global access (the rehearsal), and again
+// after it.
+constexpr int kRankMax = 384;
+template <bool kFused, int kKeys>
+__global__ void __launch_bounds__(kKeys + 32)
 select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_cand,
               int32_t* __restrict__ sel_count, int32_t* __restrict__ sel_idx, int n_kv_heads,
               int n_cap, int cap_blocks, int n_layers, int32_t* status, ChainParams ch) {
   extern __shared__ uint32_t sel_smem[];       // the head's scores [n_cap] (fp32), then their keys, each padded to a multiple of 128
-  static_assert(kSelThreads == 256, "eight warps");
-  __shared__ __align__(16) int warp_tot[2][kSelThreads / 32];
-  __shared__ float sh_thetas[8];               // the densities of the cluster's heads (written by their CTAs)
-  __shared__ float red_f[3 * (kSelThreads / 32)];
+  constexpr int kWarps = kKeys / 32;
+  __shared__ int warp_tot[2][kWarps];
+  __shared__ float sh_thetas[2][8];            // the densities of the cluster's heads (written by their CTAs), one set per pass
+  __shared__ __align__(8) uint64_t sh_bar[2];  // a pass's densities have arrived
+  __shared__ float red_m[kWarps], red_z[kWarps], red_e[kWarps];
   __shared__ int sh_count;
-  __shared__ double sh_brem, sh_rest;
-  __shared__ int sh_no_hist;
-  __shared__ float dummy_sc[32];
-  __shared__ __align__(16) uint32_t dummy_key[128];
-  const int g = blockIdx.x, unit = blockIdx.y, tid = threadIdx.x;
+  const int g = blockIdx.x, unit = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool control = warp == kWarps;
+  auto smem = [](const void* x) { return uint32_t(__cvta_generic_to_shared(x)); };
   // A peer's shared memory may be written only once that peer runs: every CTA says so here, and waits for
   // the others just ahead of its first remote store.
-  if constexpr (kFused) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+  if constexpr (kFused) {
+    if (control && lane < 2) {
+      const uint32_t bytes = 4u * uint32_t(n_kv_heads), bar = smem(sh_bar + lane);
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+    }
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  }
   grid_launch_dependents();
   const int n_real = min(n_cand[unit / n_layers], n_cap);
+  const bool ranked = n_real <= min(kRankMax, kKeys);
   const float* s = scores + (size_t(unit) * n_kv_heads + g) * n_cap;
+  int32_t* out = sel_idx + (size_t(unit) * n_kv_heads + g) * cap_blocks;
+  float* sc = reinterpret_cast<float*>(sel_smem);
+  uint32_t* keys = sel_smem + (n_cap + 127) / 128 * 128;
 #pragma unroll 1
   for (int pass = 0; pass < 2; ++pass) {
     asm volatile("" : "+r"(pass));             // one body for both passes
     const bool real = pass != 0;
     if (real) grid_dependency_wait();          // scores / densities / counts come from the stream's previous kernels
     const int n = real ? n_real : min(n_real, 32);
-    float* sc = real ? reinterpret_cast<float*>(sel_smem) : dummy_sc;
-    uint32_t* keys = real ? sel_smem + (n_cap + 127) / 128 * 128 : dummy_key;
     const int n4 = (n + 127) / 128 * 32;       // 16-byte groups of keys, padded for the search
-    // the scores are fetched once, by all threads at a time; density and selection read them from here
-    for (int i = tid; i < 4 * n4; i += kSelThreads) {
-      uint32_t key = 0u;
-      if (i < n) {
-        const float x = real ? s[i] : float(i) * 0.03f;
-        sc[i] = x;
-        key = score_key(x);
+    const int seq = unit, layer = ch.layer0;   // kFused: one layer per call
+    double* st = ch.state + size_t(seq) * (1 + 2 * ch.L);
+    double b_rem = 0.0, rest = 0.0;
+    int no_hist = 0;
+    if (!control) {
+      // the scores are fetched once, by all threads at a time; density and selection read them from here
+      float m = -INFINITY;
+      for (int i0 = tid; i0 < 4 * n4; i0 += 4 * kKeys) {
+        float x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u * kKeys;
+          x[u] = i < n ? (real ? s[i] : float(i) * 0.03f) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u * kKeys;
+          if (u > 0 && i >= 4 * n4) break;
+          if (kFused && i < n) { sc[i] = x[u]; m = fmaxf(m, ch.beta * x[u]); }
+          keys[i] = i < n ? score_key(x[u]) : 0u;
+        }
       }
-      keys[i] = key;
+      if (kFused && warp * 32 < n) {           // Eq. 11 over this warp's scores, about the warp's own maximum
+        m = warp_max_redux(m);
+        float z = 0.f, e_x = 0.f;
+#pragma unroll 2
+        for (int i = tid; i < n; i += kKeys) {
+          const float x = ch.beta * sc[i] - m, e = expf(x);
+          z += e;
+          e_x = fmaf(e, x, e_x);
+        }
+        z = warp_sum(z);
+        e_x = warp_sum(e_x);
+        if (lane == 0) { red_m[warp] = m; red_z[warp] = z; red_e[warp] = e_x; }
+      }
+    } else if constexpr (kFused) {
+      // The old state: the mean densities of the deeper layers that have a history (a lane per layer, then a
+      // butterfly over the lanes).  Every CTA reads it before it hands out its density, CTA 0 writes it after all have.
+      b_rem = real && layer > 0 ? st[0] : double(ch.L) * double(ch.k_blocks);
+      for (int j = layer + 1 + lane; j < ch.L; j += 32) {
+        const double cnt = real ? st[1 + ch.L + j] : 2.0;
+        if (cnt > 0.0) rest += (real ? st[1 + j] : 1.0) / cnt; else ++no_hist;
+      }
+#pragma unroll 1
+      for (int o = 16; o > 0; o >>= 1) rest += __shfl_xor_sync(0xffffffffu, rest, o);
+      b_rem = __shfl_sync(0xffffffffu, b_rem, 0);       // has arrived
+      no_hist = __reduce_add_sync(0xffffffffu, no_hist);
     }
-    int c;
-    if constexpr (kFused) {
-      cg::cluster_group cluster = cg::this_cluster();
-      const int seq = unit;                      // one layer per call: unit == sequence
-      const int layer = ch.layer0;
-      double* st = ch.state + size_t(seq) * (1 + 2 * ch.L);
-      // The old state is read by every CTA before the cluster barrier, written by CTA 0 after it.
-      // Warp 1 adds up the mean densities of the deeper layers that have a history (a lane per
-      // layer, then a butterfly over the lanes) while the scores arrive.
-      if (tid >= 32 && tid < 64) {
-        const int lane = tid - 32;
-        double part = 0.0;
-        int none = 0;
-        for (int j = layer + 1 + lane; j < ch.L; j += 32) {
-          const double cnt = real ? st[1 + ch.L + j] : 2.0;
-          if (cnt > 0.0) part += (real ? st[1 + j] : 1.0) / cnt; else ++none;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          part += __shfl_xor_sync(0xffffffffu, part, o);
-          none += __shfl_xor_sync(0xffffffffu, none, o);
-        }
-        if (lane == 0) {
-          sh_brem = layer == 0 || !real ? double(ch.L) * double(ch.k_blocks) : st[0];
-          sh_rest = part;
-          sh_no_hist = none;
-        }
+    __syncthreads();
+    if constexpr (kFused) if (!real) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    int rank = 0;
+    if (!control) {
+      if (ranked && warp * 32 < n) rank = rank_of(keys[tid], tid, keys, n);
+    } else if constexpr (kFused) {
+      const size_t uh = size_t(unit) * n_kv_heads + g;
+      float th_own;
+      if (ch.theta_in && real) {
+        th_own = ch.theta_in[uh];
+      } else {                                 // the warps' sums, moved to the common maximum
+        const bool on = lane < kWarps && lane * 32 < n;
+        const float m = on ? red_m[lane] : -INFINITY, top = warp_max_redux(m);
+        const float x = on ? m - top : 0.f, f = on ? expf(x) : 0.f, zw = on ? red_z[lane] : 0.f;
+        float z = f * zw, e_x = on ? f * fmaf(zw, x, red_e[lane]) : 0.f;
+        z = warp_sum(z);
+        e_x = warp_sum(e_x);
+        th_own = n > 0 ? fmaxf(logf(z) - e_x / z, 0.f) : 0.f;
+        if (lane == 0 && !ch.theta_in && ch.theta_out && real) ch.theta_out[uh] = th_own;
       }
-      __syncthreads();
-      // this head's density, by the whole CTA; handed to every CTA of the cluster (one per KV head)
-      // by remote stores ahead of the cluster barrier, so that nobody reads a peer's memory after it
-      // and no CTA has to wait for its peers before it leaves
-      {
-        const size_t uh = size_t(unit) * n_kv_heads + g;
-        const float th = ch.theta_in && real ? ch.theta_in[uh] : block_entropy<kSelThreads>(sc, n, ch.beta, red_f);
-        if (tid == 0 && !ch.theta_in && ch.theta_out && real) ch.theta_out[uh] = th;
-        if (!real) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-        if (tid < n_kv_heads) cluster.map_shared_rank(sh_thetas, unsigned(tid))[g] = th;
+      const uint32_t bar = smem(sh_bar + pass);
+      if (lane < n_kv_heads) {
+        uint32_t dst, far;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(smem(&sh_thetas[pass][g])), "r"(lane));
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(far) : "r"(bar), "r"(lane));
+        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+                     ::"r"(dst), "r"(__float_as_uint(th_own)), "r"(far) : "memory");
       }
-      asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-      asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-      if (tid == 0) {
-        float th_h[8];
-#pragma unroll
-        for (int h2 = 0; h2 < 8; ++h2) th_h[h2] = h2 < n_kv_heads ? sh_thetas[h2] : 0.f;
-        double sum = 0.0;
-#pragma unroll
-        for (int h2 = 0; h2 < 8; ++h2) sum += double(th_h[h2]);
-        const double th = sum / double(n_kv_heads);
-        const double b_rem = sh_brem, rest_hist = sh_rest;
-        const int no_hist = sh_no_hist;
-        Grant gr{0, 0.0};
-        if (n > 0) {
-          // layers without history count with this layer's density; with every layer in the call
-          // (L == 1) there is no deeper layer and both theta-bar readings coincide
-          const double rest = rest_hist + double(no_hist) * th;
-          gr = grant_layer(th, rest, b_rem, ch.L - layer, n, ch.cap_blocks);
-        }
+      bool here = false;
+      for (uint32_t i = 0; i < (1u << 20) && !here; ++i) {        // bounded
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\tselp.b32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(bar) : "memory");
+        here = ok != 0;
+      }
+      if (!here && lane == 0) set_status(status, ACTQKV_DEV_TIMEOUT);
+      double sum = 0.0;
+      for (int h = 0; h < n_kv_heads; ++h) sum += double(sh_thetas[pass][h]);
+      const double th = sum / double(n_kv_heads);
+      Grant gr{0, 0.0};
+      // layers without history count with this layer's density; with every layer in the call
+      // (L == 1) there is no deeper layer and both theta-bar readings coincide
+      if (n > 0) gr = grant_layer(th, rest + double(no_hist) * th, b_rem, ch.L - layer, n, ch.cap_blocks);
+      if (lane == 0) {
         sh_count = real ? gr.c : 5;
         if (g == 0 && real) {
           st[0] = n > 0 ? b_rem - double(gr.c) : b_rem;
@@ -333,47 +391,54 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
           if (ch.budget_real) ch.budget_real[unit] = float(gr.real);
         }
       }
-      __syncthreads();
-      c = sh_count;
     } else {
-      c = real ? sel_count[unit] : 5;
-      if (real && (c < 0 || c > min(cap_blocks, n))) {
-        if (tid == 0) set_status(status, ACTQKV_DEV_BAD_SELECTION);
-        c = max(0, min(c, min(cap_blocks, n)));
+      if (lane == 0) {
+        int c = real ? sel_count[unit] : 5;
+        if (real && (c < 0 || c > min(cap_blocks, n))) {
+          set_status(status, ACTQKV_DEV_BAD_SELECTION);
+          c = max(0, min(c, min(cap_blocks, n)));
+        }
+        sh_count = c;
       }
-      __syncthreads();                           // the keys are written
     }
-    int32_t* out = sel_idx + (size_t(unit) * n_kv_heads + g) * cap_blocks;
-    if (real)
-      for (int i = c + tid; i < cap_blocks; i += kSelThreads) out[i] = -1;
-    if (c >= n) {
+    __syncthreads();
+    const int c = sh_count;
+    if (control) {
       if (real)
-        for (int i = tid; i < min(n, c); i += kSelThreads) out[i] = i;
+        for (int i = max(c, 0) + lane; i < cap_blocks; i += 32) out[i] = -1;
+    } else if (ranked) {
+      const bool take = tid < n && rank < c;
+      const uint32_t votes = __ballot_sync(0xffffffffu, take);
+      if (lane == 0) warp_tot[0][warp] = __popc(votes);
+      key_sync<kKeys>();
+      const int pos = __reduce_add_sync(0xffffffffu, lane < warp ? warp_tot[0][lane] : 0) + __popc(votes & ((1u << lane) - 1u));
+      if (take && pos < cap_blocks && real) out[pos] = tid;
+    } else if (c >= n) {
+      if (real)
+        for (int i = tid; i < min(n, c); i += kKeys) out[i] = i;
     } else if (c > 0) {
       // ---- the largest threshold that at least c keys reach; done early when exactly c do
       int at = n;                                // keys >= thr
-      const uint32_t thr = search_cth(c, keys, n4, warp_tot, at);
+      const uint32_t thr = search_cth<kKeys>(c, keys, n4, warp_tot, at);
       // at > c: thr is the c-th largest key itself and at - c too many keys equal it; of those the first
       // by index are admitted
       int need_eq = n;
       if (at > c) {
         int above = 0;
-        for (int i = tid; i < n; i += kSelThreads) above += keys[i] > thr;
+        for (int i = tid; i < n; i += kKeys) above += keys[i] > thr;
         above = __reduce_add_sync(0xffffffffu, above);
-        __syncthreads();
-        if ((tid & 31) == 0) warp_tot[0][tid >> 5] = above;
-        __syncthreads();
-        need_eq = c;
-        for (int w = 0; w < kSelThreads / 32; ++w) need_eq -= warp_tot[0][w];
-        __syncthreads();
+        key_sync<kKeys>();
+        if (lane == 0) warp_tot[0][warp] = above;
+        key_sync<kKeys>();
+        need_eq = c - __reduce_add_sync(0xffffffffu, lane < kWarps ? warp_tot[0][lane] : 0);
       }
-      const int per = (n + kSelThreads - 1) / kSelThreads;
+      const int per = (n + kKeys - 1) / kKeys;
       const int i0 = min(n, tid * per), i1 = min(n, i0 + per);
-      int tot, eq_before = 0;
+      int eq_before = 0;
       if (at > c) {
         int eq = 0;
         for (int i = i0; i < i1; ++i) eq += keys[i] == thr;
-        eq_before = block_exclusive_scan(eq, warp_tot[0], &tot);
+        eq_before = key_exclusive_scan<kKeys>(eq, warp_tot[0]);
       }
       // compacted in ascending block order
       int cnt = 0, e = eq_before;
@@ -381,7 +446,7 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
         const uint32_t x = keys[i];
         cnt += at > c ? (x > thr || (x == thr && e++ < need_eq)) : x >= thr;
       }
-      int pos = block_exclusive_scan(cnt, warp_tot[0], &tot);
+      int pos = key_exclusive_scan<kKeys>(cnt, warp_tot[0]);
       e = eq_before;
       for (int i = i0; i < i1; ++i) {
         const uint32_t x = keys[i];
@@ -408,7 +473,12 @@ int launch_cutoff(const actqkv_config* cfg, const Batch& b, const float* scores,
   p.thetabar_mode = cfg->thetabar_mode; p.beta = cfg->beta;
   const size_t sm_sel = (size_t(cfg->n_cap) + 127) / 128 * 128 * 8;        // scores and keys
   const bool fused = b.n_layers == 1 && cfg->n_kv_heads <= 8 && cfg->cap_blocks > 0;
-  auto kern = fused ? select_kernel<true> : select_kernel<false>;
+  // 512 key threads where 256 would hold several candidates each and the CTAs have the SMs to themselves; a grid that fills
+  // the SMs keeps the narrow form, which becomes resident beside two CTAs of the streaming scores (288 threads x 56
+  // registers; 16 sequences of 32k-131k tokens, a decode step of two layers: 168 us).
+  const bool wide = cfg->n_cap > 256 && b.units() * cfg->n_kv_heads <= kNumSMs / 2;
+  auto kern = fused ? (wide ? select_kernel<true, 512> : select_kernel<true, 256>)
+                    : (wide ? select_kernel<false, 512> : select_kernel<false, 256>);
   if (sm_sel > 40 * 1024 &&
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm_sel)) != cudaSuccess)
     return ACTQKV_ERR_LAUNCH;
@@ -436,11 +506,11 @@ int launch_cutoff(const actqkv_config* cfg, const Batch& b, const float* scores,
     if (cudaLaunchKernelEx(&lcc, cutoff_chain_kernel, p) != cudaSuccess) return ACTQKV_ERR_LAUNCH;
     if (cfg->cap_blocks == 0) return ACTQKV_OK;
   }
-  static std::atomic<bool> carved[2][kMaxDevices];
-  prefer_max_shared(kern, carved[fused]);
+  static std::atomic<bool> carved[4][kMaxDevices];
+  prefer_max_shared(kern, carved[2 * wide + fused]);
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3(cfg->n_kv_heads, b.units(), 1);
-  lc.blockDim = dim3(kSelThreads, 1, 1);
+  lc.blockDim = dim3((wide ? 512 : 256) + 32, 1, 1);
   lc.dynamicSmemBytes = sm_sel;
   lc.stream = st;
   cudaLaunchAttribute attr[2];

@@ -46,3 +46,38 @@ def test_selection_edges(layers, n, kind):
             assert 1 <= k <= c
             for g in range(0, 8, 3):
                 assert got[u][g] == pick(host[u][g], k) + [-1] * (c - k), (u, g, k)
+
+
+@pytest.mark.parametrize("seqs", [1, 12])            # up to 9 sequences of 8 KV heads take a thread per candidate up to 512
+@pytest.mark.parametrize("n", [5, 32, 33, 129, 256, 257, 384, 385, 511, 513, 1500])
+def test_density_and_selection_of_one_layer(seqs, n):
+    """Density, count and set of one layer from its own scores: lengths at the edges of a warp, of the ranked range and of
+    the key threads.  The density is a sum of n fp32 terms about 1: n * 2^-24 of it, and a few roundings of exp and ln."""
+    import torch
+    from paper_2502_13542_b200 import binding as B
+    L, c, beta = 3, min(n, 40), 8.0
+    spec = wl.llama3_8b_layer().replace(n_layers=L, k_blocks=c, cap_blocks=c, n_kv_heads=8)
+    cfg = B.make_config(spec, n_cap=n, beta=beta)
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    table = torch.randn(seqs, 8, n, 4, 128, device="cuda", generator=gen).bfloat16()
+    norms = 1.0 / table.float().norm(dim=-1)
+    probe = torch.randn(seqs, 8, 128, device="cuda", generator=gen)
+    n_cand = torch.full((seqs,), n, dtype=torch.int32, device="cuda")
+    n_cand[-1] = max(1, n - 3)
+    state = torch.zeros(seqs, 1 + 2 * L, dtype=torch.float64, device="cuda")
+    scores, theta = torch.zeros(seqs, 8, n, device="cuda"), torch.zeros(seqs, 8, device="cuda")
+    sel = torch.full((seqs, 8, c), -7, dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(seqs, dtype=torch.int32, device="cuda")
+    for layer in range(L):
+        B.score_select(cfg, B.Batch(seqs, 1, layer), probe, table, norms, n_cand, state, scores, theta, sel, cnt)
+        torch.cuda.synchronize()
+        for u in range(seqs):
+            m = int(n_cand[u])
+            x = beta * scores[u, :, :m].double()
+            w = torch.softmax(x, dim=-1)
+            want = torch.special.entr(w).sum(-1)
+            assert torch.allclose(theta[u].double(), want, rtol=(n + 16) * 2.0 ** -24, atol=1e-6)
+            k = int(cnt[u])
+            assert 1 <= k <= min(c, m)
+            for g in range(8):
+                assert sel[u, g].tolist() == pick(scores[u, g, :m].tolist(), k) + [-1] * (c - k)
