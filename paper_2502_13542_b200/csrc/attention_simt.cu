@@ -4,18 +4,22 @@
 // dim / page size / alignment; serves fp32 caches and what the tensor-core kernels do not take.
 //
 // One CTA = 32 rows of one KV head: the (token, query head) pairs of the group, row = token * G + head,
-// so that K and V are read once per group.  Keys go through shared memory in chunks of 64, as fp32.
-// Thread (ty, tx), ty = 0..7, tx = 0..15: rows 4 ty .. + 3; in the Q K^T phase keys tx + 16 j, in the P V
-// phase channels 4 tx .. + 3 (and + 64): 4 x 4 register tiles, eight 16-byte shared loads per 64 FMAs, and
-// the 16 lanes that share a row lie in one half-warp, so that a row's maximum and sum are shuffles.
-// Softmax is the usual running-max / running-sum recurrence in base 2.
+// so that K and V are read once per group.  Keys go through shared memory in chunks, as fp32, two buffers: a producer
+// warp looks the keys up (position -> page table, behind the selection's entries), brings chunk c + 1 and waits for it while
+// the four compute warps work on chunk c; one CTA barrier per chunk.
+// A compute warp has 8 rows; its lanes have one key each (two at D = 64) in Q K^T and D / 32 channels each in P V.  Bound
+// by the shared-memory bandwidth: Q and P are read by broadcast, one 128-byte wavefront per 16-byte load, and K and V
+// by 32 lanes apart, 16 wavefronts per 64 FMAs of a warp (with 4 rows x 4 keys per thread, 16 lanes to a row, it was 32).
 //
-// The kernel is bound by latency on small steps: few tiles, each a serial walk over the keys.  So the
-// chunks are cut over the CTAs of a cluster (chunk c goes to rank c % n), the partial results are merged
-// through distributed shared memory, and a key's place in the cache (two dependent look-ups) is found one
-// chunk ahead of its use.  A window of 256 tokens x 4 heads over 1,400 keys (D = 64, fp32) took 166 us
-// with 16 rows of one head per CTA and no cut; a prompt of 16 such windows 3,826 us, now 1,503 us.
+// The initial tokens, the local past and the step's own tokens come first and the selected blocks last: the former are
+// known before this step's selection exists, so their chunks run ahead of the dependency wait (programmatic dependent
+// launch).  Few tiles: the chunks are cut over the CTAs of a cluster (chunk c goes to rank c % n) and the partial
+// results are merged through distributed shared memory.
+// A window of 256 tokens x 4 heads over 1,400 keys (D = 64, fp32), launches one behind the other: 28.7 us with all threads
+// staging each chunk between two barriers and every key behind the wait, 22.3 us like this (25.3 us with a producer lane
+// per 16 bytes, which spent 6k clk a chunk on addresses); a prompt of 16 such windows 663 -> 565 us.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "stages.cuh"
@@ -25,15 +29,16 @@ using namespace actqkv;
 namespace {
 
 constexpr int kRows = 32;
-constexpr int kChunk = 64;
-constexpr int kThreads = 128;
+constexpr int kComputeWarps = 4, kRowsPerWarp = kRows / kComputeWarps;
+constexpr int kThreads = 32 * (kComputeWarps + 1);
 constexpr int kMaxSplits = 8;
 
 template <int D> struct Smem {
-  static constexpr int kKStride = D + 4;             // floats; 16 consecutive keys at one channel vector hit distinct banks
+  static constexpr int kChunk = D == 64 ? 64 : 32;   // keys; two CTAs per SM
+  static constexpr int kKStride = D + 4;             // floats; 32 consecutive keys at one channel vector hit distinct banks
   static constexpr int kPStride = kChunk + 4;
-  static constexpr int kQ = 0, kK = kQ + kRows * D, kV = kK + kChunk * kKStride, kP = kV + kChunk * D,
-                       kFloats = kP + kRows * kPStride;
+  static constexpr int kKV = kChunk * (kKStride + D);                   // one buffer: K, then V
+  static constexpr int kQ = 0, kBuf = kQ + kRows * D, kP = kBuf + 2 * kKV, kFloats = kP + kRows * kPStride;
   static constexpr int kBytes = kFloats * 4;
 };
 
@@ -67,32 +72,25 @@ __device__ __forceinline__ float ld_peer(const float* local, uint32_t rank) {
   asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
   return v;
 }
-__device__ __forceinline__ float half_warp_max(float v) {
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ float half_warp_sum(float v) {
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+__device__ __forceinline__ void cp_async16(float* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(uint32_t(__cvta_generic_to_shared(dst))), "l"(src) : "memory");
 }
 
 template <typename T, typename TO, int D>
-__global__ void __launch_bounds__(kThreads) attention_simt_kernel(SimtParams p) {
+__global__ void __launch_bounds__(kThreads, 2) attention_simt_kernel(SimtParams p) {
   using S = Smem<D>;
+  constexpr int kChunk = S::kChunk, KPL = kChunk / 32, CPL = D / 32;   // keys and channels per lane
+  constexpr int VN = Vec16<T>::N, VPR = D / VN, R = kRowsPerWarp;
   extern __shared__ __align__(16) float sm[];
-  float *Qs = sm + S::kQ, *Ks = sm + S::kK, *Vs = sm + S::kV, *Ps = sm + S::kP;
-  __shared__ int64_t place[2][kChunk];                // element offset of a key in its cache pool or in the step; -1: none
+  float *Qs = sm + S::kQ, *Ps = sm + S::kP;
   __shared__ float part_m[kRows], part_l[kRows];
 
   grid_launch_dependents();          // the append makes its loads while this kernel runs
   const uint32_t rank = p.n_splits > 1 ? cluster_rank() : 0u;
   const int tile = blockIdx.x / p.n_splits, g = blockIdx.y, unit = blockIdx.z;
   const int G = p.group, seq = unit / p.n_layers, layer_local = unit - seq * p.n_layers;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nt = p.a.n_tokens, n_rows = nt * G;
-  constexpr int VN = Vec16<T>::N, VPR = D / VN, NC = D / 64;      // NC: column quads of a thread in the P V phase
 
   const Geometry geo = make_geometry(p.a.pos0[seq], p.n_init, p.block, p.n_local_prev);
   const T* qb = static_cast<const T*>(p.a.q) + size_t(unit) * nt * p.n_q_heads * D;
@@ -108,212 +106,277 @@ __global__ void __launch_bounds__(kThreads) attention_simt_kernel(SimtParams p) 
 #pragma unroll
     for (int e = 0; e < VN; ++e) Qs[r * D + cv * VN + e] = qf[e];
   }
-  grid_dependency_wait();            // the selection comes from the stream's previous kernel
 
-  int c = p.a.sel_count ? p.a.sel_count[unit] : 0;
-  if (c < 0 || c > p.cap_blocks || c > geo.n_cand) {
-    if (tid == 0) set_status(p.a.status, ACTQKV_DEV_BAD_SELECTION);
-    c = max(0, min(c, min(p.cap_blocks, geo.n_cand)));
-  }
-  const int32_t* sel = p.a.sel_idx + (size_t(unit) * p.n_kv_heads + g) * p.cap_blocks;
-  const int sel_len = c * p.block;
-  const int64_t n_past = int64_t(geo.init_len) + sel_len + (geo.p0 - geo.local_start);
-  const size_t page_elems = size_t(p.n_kv_heads) * p.page_tokens * D;
-  const T* kp = static_cast<const T*>(p.a.k_pages) + size_t(layer_local) * p.n_phys_pages * page_elems;
-  const T* vp = static_cast<const T*>(p.a.v_pages) + size_t(layer_local) * p.n_phys_pages * page_elems;
-  const int32_t* pt = p.a.page_table + size_t(seq) * p.max_pages;
-  const T* kw = static_cast<const T*>(p.a.k_win) + size_t(unit) * nt * p.n_kv_heads * D;
-  const T* vw = static_cast<const T*>(p.a.v_win) + size_t(unit) * nt * p.n_kv_heads * D;
-
+  // ---- the key stream: [initial | local past | step's tokens], filled up to whole chunks, then the selected blocks
+  const int64_t n_past = int64_t(geo.init_len) + (geo.p0 - geo.local_start);
   const int last_row = min(n_rows, (tile + 1) * kRows) - 1;
-  const int64_t n_keys = n_past + last_row / G + 1;
-  // the place of key i: an offset into the cache pool (i < n_past) or into the step's own keys
-  auto find = [&](int64_t i) -> int64_t {
-    if (i >= n_keys) return -1;
-    if (i >= n_past) return ((i - n_past) * p.n_kv_heads + g) * D;
-    int64_t tok;
-    if (i < geo.init_len) {
-      tok = i;
-    } else if (i < geo.init_len + sel_len) {
-      const int r = int(i - geo.init_len), blk = sel[r / p.block];
-      if (blk < 0 || blk >= geo.n_cand) {
-        set_status(p.a.status, ACTQKV_DEV_BAD_SELECTION);
+  const int64_t n_early = n_past + last_row / G + 1;
+  const int64_t early = (n_early + kChunk - 1) / kChunk;               // chunks ahead of the wait
+  int64_t total = early;                                               // all chunks, known after it
+  int sel_len = 0;
+  bool open = false;
+  // Every warp that comes to the selected blocks takes the wait itself (it is the launch dependency, so it always ends).
+  auto wait_selection = [&]() {
+    grid_dependency_wait();
+    int c = p.a.sel_count ? p.a.sel_count[unit] : 0;
+    if (c < 0 || c > p.cap_blocks || c > geo.n_cand) {
+      if (tid == 0) set_status(p.a.status, ACTQKV_DEV_BAD_SELECTION);
+      c = max(0, min(c, min(p.cap_blocks, geo.n_cand)));
+    }
+    sel_len = c * p.block;
+    total = early + (sel_len + kChunk - 1) / kChunk;
+    open = true;
+  };
+  __syncthreads();                                     // Q is written
+
+  float m[R], l[R], o[R][CPL];                         // l: this lane's share of the row's sum
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    m[r] = -INFINITY; l[r] = 0.f;
+#pragma unroll
+    for (int q = 0; q < CPL; ++q) o[r][q] = 0.f;
+  }
+
+  if (warp == kComputeWarps) {
+    // =========================== producer ===========================
+    const int32_t* sel = p.a.sel_idx + (size_t(unit) * p.n_kv_heads + g) * p.cap_blocks;
+    const size_t page_elems = size_t(p.n_kv_heads) * p.page_tokens * D;
+    const T* kp = static_cast<const T*>(p.a.k_pages) + size_t(layer_local) * p.n_phys_pages * page_elems;
+    const T* vp = static_cast<const T*>(p.a.v_pages) + size_t(layer_local) * p.n_phys_pages * page_elems;
+    const int32_t* pt = p.a.page_table + size_t(seq) * p.max_pages;
+    const T* kw = static_cast<const T*>(p.a.k_win) + size_t(unit) * nt * p.n_kv_heads * D;
+    const T* vw = static_cast<const T*>(p.a.v_win) + size_t(unit) * nt * p.n_kv_heads * D;
+    // the place of key i: its element offset in the cache pool or (n_past <= i < n_early) in the step's own keys; -1: none
+    auto find = [&](int64_t i) -> int64_t {
+      int64_t tok;
+      if (i >= early * kChunk) {
+        const int64_t r = i - early * kChunk;
+        if (r >= sel_len) return -1;
+        const int blk = sel[int(r) / p.block];
+        if (blk < 0 || blk >= geo.n_cand) {
+          set_status(p.a.status, ACTQKV_DEV_BAD_SELECTION);
+          return -1;
+        }
+        tok = int64_t(p.n_init) + int64_t(blk) * p.block + int(r) % p.block;
+      } else {
+        if (i >= n_early) return -1;
+        if (i >= n_past) return ((i - n_past) * p.n_kv_heads + g) * D;
+        tok = i < geo.init_len ? i : geo.local_start + (i - geo.init_len);
+      }
+      const int64_t lp = tok / p.page_tokens;
+      const int phys = lp < p.max_pages ? pt[lp] : -1;
+      if (phys < 0 || phys >= p.n_phys_pages) {
+        set_status(p.a.status, ACTQKV_DEV_BAD_PAGE);
         return -1;
       }
-      tok = int64_t(p.n_init) + int64_t(blk) * p.block + r % p.block;
-    } else {
-      tok = geo.local_start + (i - geo.init_len - sel_len);
-    }
-    const int64_t lp = tok / p.page_tokens;
-    const int phys = lp < p.max_pages ? pt[lp] : -1;
-    if (phys < 0 || phys >= p.n_phys_pages) {
-      set_status(p.a.status, ACTQKV_DEV_BAD_PAGE);
-      return -1;
-    }
-    return (int64_t(phys) * p.n_kv_heads + g) * p.page_tokens * D + (tok - lp * p.page_tokens) * D;
-  };
-
-  float m[4], l[4], o[4][NC][4];
-  int lim[4];                                          // this thread's rows see the step's tokens [0, lim)
+      return (int64_t(phys) * p.n_kv_heads + g) * p.page_tokens * D + (tok - lp * p.page_tokens) * D;
+    };
+    struct Places { int64_t at[KPL]; };
+    auto look_up = [&](int64_t c) {
+      Places x;
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    m[r] = -INFINITY; l[r] = 0.f;
-    lim[r] = (tile * kRows + ty * 4 + r) / G + 1;
+      for (int j = 0; j < KPL; ++j) x.at[j] = find(c * kChunk + 32 * j + lane);
+      return x;
+    };
+    // Two lanes per key, 16 keys at a time: whole 32-byte sectors, and no address arithmetic between a row's copies.
+    auto bring = [&](int64_t c, const Places& x, float* Ks) {
+      float* Vs = Ks + kChunk * S::kKStride;
+      const int half = lane & 1;
 #pragma unroll
-    for (int q = 0; q < NC; ++q)
+      for (int j = 0; j < 2 * KPL; ++j) {
+        const int in = 16 * (j & 1) + (lane >> 1), row = 32 * (j >> 1) + in;
+        const int64_t at = __shfl_sync(0xffffffffu, x.at[j >> 1], in);
+        const bool past = c >= early || c * kChunk + row < n_past;
+        const T *ks = (past ? kp : kw) + at + half * VN, *vs = (past ? vp : vw) + at + half * VN;
+        float *kd = Ks + row * S::kKStride + half * VN, *vd = Vs + row * D + half * VN;
+        if (at < 0) {
+#pragma unroll 1
+          for (int e = 0; e < D; e += 2 * VN)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) o[r][q][e] = 0.f;
-  }
-
-  const int64_t step = int64_t(kChunk) * p.n_splits;
-  int64_t kc = int64_t(kChunk) * rank;
-  if (tid < kChunk) place[0][tid] = find(kc + tid);
-  for (int buf = 0; kc < n_keys; kc += step, buf ^= 1) {
-    __syncthreads();                                   // the places are written, the last chunk's readers are done
-    if (tid >= kThreads - kChunk) place[buf ^ 1][tid - (kThreads - kChunk)] = find(kc + step + tid - (kThreads - kChunk));
-    // ---- stage the chunk as fp32, a batch of loads in flight per thread
-    constexpr int kLoads = kChunk * VPR / kThreads, kBatch = kLoads < 4 ? kLoads : 4;
+            for (int f = 0; f < VN; f += 4)
+              *reinterpret_cast<float4*>(kd + e + f) = *reinterpret_cast<float4*>(vd + e + f) = make_float4(0.f, 0.f, 0.f, 0.f);
+        } else if constexpr (sizeof(T) == 4) {
 #pragma unroll
-    for (int b0 = 0; b0 < kLoads; b0 += kBatch) {
-      uint4 kr[kBatch], vr[kBatch];
+          for (int e = 0; e < D; e += 2 * VN) {
+            cp_async16(kd + e, ks + e);
+            cp_async16(vd + e, vs + e);
+          }
+        } else {
+          constexpr int kBatch = 4;
 #pragma unroll
-      for (int b = 0; b < kBatch; ++b) {
-        const int i = (b0 + b) * kThreads + tid, row = i / VPR, cv = i - row * VPR;
-        const int64_t at = place[buf][row];
-        kr[b] = vr[b] = make_uint4(0, 0, 0, 0);
-        if (at >= 0) {
-          const bool past = kc + row < n_past;
-          kr[b] = __ldg(reinterpret_cast<const uint4*>((past ? kp : kw) + at + cv * VN));
-          vr[b] = __ldg(reinterpret_cast<const uint4*>((past ? vp : vw) + at + cv * VN));
+          for (int e0 = 0; e0 < D; e0 += 2 * VN * kBatch) {
+            uint4 kr[kBatch], vr[kBatch];
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+              kr[u] = __ldg(reinterpret_cast<const uint4*>(ks + e0 + u * 2 * VN));
+              vr[u] = __ldg(reinterpret_cast<const uint4*>(vs + e0 + u * 2 * VN));
+            }
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+              float kf[VN], vf[VN];
+              Vec16<T>::unpack(kr[u], kf);
+              Vec16<T>::unpack(vr[u], vf);
+#pragma unroll
+              for (int f = 0; f < VN; f += 4) {
+                const int e = e0 + u * 2 * VN + f;
+                *reinterpret_cast<float4*>(kd + e) = make_float4(kf[f], kf[f + 1], kf[f + 2], kf[f + 3]);
+                *reinterpret_cast<float4*>(vd + e) = make_float4(vf[f], vf[f + 1], vf[f + 2], vf[f + 3]);
+              }
+            }
+          }
         }
       }
+    };
+    int64_t c = rank;
+    if (c >= early) wait_selection();
+    Places x = look_up(c);
+    for (int buf = 0; c < total; buf ^= 1) {
+      bring(c, x, sm + S::kBuf + buf * S::kKV);
+      c += p.n_splits;
+      const bool known = c < early || open;
+      if (known && c < total) x = look_up(c);          // while the copies fly
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncthreads();                                 // the chunk is there, and the other buffer has been read
+      if (!known) {
+        wait_selection();
+        if (c < total) x = look_up(c);
+      }
+    }
+  } else {
+    // =========================== compute ===========================
+    int lim[R];                                        // the warp's rows see the step's tokens [0, lim)
 #pragma unroll
-      for (int b = 0; b < kBatch; ++b) {
-        const int i = (b0 + b) * kThreads + tid, row = i / VPR, cv = i - row * VPR;
-        float kf[VN], vf[VN];
-        Vec16<T>::unpack(kr[b], kf);
-        Vec16<T>::unpack(vr[b], vf);
+    for (int r = 0; r < R; ++r) lim[r] = min((tile * kRows + warp * R + r) / G, last_row / G) + 1;
+    const float* q_rows = Qs + warp * R * D;
+    float* p_rows = Ps + warp * R * S::kPStride;
+    int64_t c = rank;
+    for (int buf = 0;; buf ^= 1, c += p.n_splits) {
+      if (c >= early && !open) wait_selection();
+      if (c >= total) break;
+      __syncthreads();                                 // the chunk is there
+      const float *Ks = sm + S::kBuf + buf * S::kKV, *Vs = Ks + kChunk * S::kKStride;
+      // ---- S = Q K^T: keys lane + 32 j
+      float s[R][KPL];
 #pragma unroll
-        for (int e = 0; e < VN; e += 4) {
-          *reinterpret_cast<float4*>(Ks + row * S::kKStride + cv * VN + e) = make_float4(kf[e], kf[e + 1], kf[e + 2], kf[e + 3]);
-          *reinterpret_cast<float4*>(Vs + row * D + cv * VN + e) = make_float4(vf[e], vf[e + 1], vf[e + 2], vf[e + 3]);
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int j = 0; j < KPL; ++j) s[r][j] = 0.f;
+#pragma unroll 2
+      for (int d = 0; d < D; d += 4) {
+        float4 kv[KPL], qv[R];
+#pragma unroll
+        for (int j = 0; j < KPL; ++j) kv[j] = *reinterpret_cast<const float4*>(Ks + (lane + 32 * j) * S::kKStride + d);
+#pragma unroll
+        for (int r = 0; r < R; ++r) qv[r] = *reinterpret_cast<const float4*>(q_rows + r * D + d);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int j = 0; j < KPL; ++j) {
+            s[r][j] = fmaf(qv[r].x, kv[j].x, s[r][j]);
+            s[r][j] = fmaf(qv[r].y, kv[j].y, s[r][j]);
+            s[r][j] = fmaf(qv[r].z, kv[j].z, s[r][j]);
+            s[r][j] = fmaf(qv[r].w, kv[j].w, s[r][j]);
+          }
+      }
+      // ---- running softmax of the warp's rows
+      // row r sees the chunk's keys [0, lim_r): all of the past, its own part of the step's tokens, the selected blocks
+      const bool window = c < early;
+      const int64_t rest = window ? n_past - c * kChunk : sel_len - (c - early) * kChunk;
+      const int past_lim = int(min(rest, int64_t(kChunk)));            // negative: behind the past
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        float mx = -INFINITY;
+        const int lim_r = window ? past_lim + (past_lim < kChunk ? lim[r] : 0) : past_lim;
+#pragma unroll
+        for (int j = 0; j < KPL; ++j) {
+          s[r][j] = lane + 32 * j < lim_r ? s[r][j] * p.scale_log2 : -INFINITY;
+          mx = fmaxf(mx, s[r][j]);
         }
-      }
-    }
-    __syncthreads();
-
-    // ---- S = Q K^T: rows 4 ty + r, keys tx + 16 j
-    float s[4][4];
+        const float m_new = fmaxf(m[r], warp_max_redux(mx));
+        const float corr = m_new == -INFINITY ? 1.f : exp2f(m[r] - m_new);
+        float sum = 0.f;
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) s[r][j] = 0.f;
-#pragma unroll 4
-    for (int d = 0; d < D; d += 4) {
-      float4 kv[4], qv[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) kv[j] = *reinterpret_cast<const float4*>(Ks + (tx + 16 * j) * S::kKStride + d);
-#pragma unroll
-      for (int r = 0; r < 4; ++r) qv[r] = *reinterpret_cast<const float4*>(Qs + (ty * 4 + r) * D + d);
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          s[r][j] = fmaf(qv[r].x, kv[j].x, s[r][j]);
-          s[r][j] = fmaf(qv[r].y, kv[j].y, s[r][j]);
-          s[r][j] = fmaf(qv[r].z, kv[j].z, s[r][j]);
-          s[r][j] = fmaf(qv[r].w, kv[j].w, s[r][j]);
+        for (int j = 0; j < KPL; ++j) {
+          const float e = m_new == -INFINITY ? 0.f : exp2f(s[r][j] - m_new);
+          p_rows[r * S::kPStride + lane + 32 * j] = e;
+          sum += e;
         }
-    }
-    // ---- running softmax of the thread's four rows
+        l[r] = l[r] * corr + sum;
+        m[r] = m_new;
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      float mx = -INFINITY;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int64_t i = kc + tx + 16 * j;
-        const bool valid = i < n_past || (i < n_keys && i - n_past < lim[r]);
-        s[r][j] = valid ? s[r][j] * p.scale_log2 : -INFINITY;
-        mx = fmaxf(mx, s[r][j]);
+        for (int q = 0; q < CPL; ++q) o[r][q] *= corr;
       }
-      const float m_new = fmaxf(m[r], half_warp_max(mx));
-      const float corr = m_new == -INFINITY ? 1.f : exp2f(m[r] - m_new);
-      float sum = 0.f;
+      __syncwarp();                                    // a row's weights are written and read by one warp
+      // ---- O += P V: channels CPL * lane ..
+#pragma unroll 2
+      for (int k = 0; k < kChunk; k += 4) {
+        float4 pv[R];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float e = m_new == -INFINITY ? 0.f : exp2f(s[r][j] - m_new);
-        Ps[(ty * 4 + r) * S::kPStride + tx + 16 * j] = e;
-        sum += e;
-      }
-      l[r] = l[r] * corr + half_warp_sum(sum);
-      m[r] = m_new;
-#pragma unroll
-      for (int q = 0; q < NC; ++q)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) o[r][q][e] *= corr;
-    }
-    __syncwarp();                                      // a row's weights are written and read by one half-warp
-    // ---- O += P V: channels 64 q + 4 tx .. + 3
-#pragma unroll 4
-    for (int k = 0; k < kChunk; k += 4) {
-      float4 pv[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) pv[r] = *reinterpret_cast<const float4*>(Ps + (ty * 4 + r) * S::kPStride + k);
-#pragma unroll
-      for (int q = 0; q < NC; ++q) {
+        for (int r = 0; r < R; ++r) pv[r] = *reinterpret_cast<const float4*>(p_rows + r * S::kPStride + k);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-          const float4 v = *reinterpret_cast<const float4*>(Vs + (k + kk) * D + 64 * q + 4 * tx);
+          float v[CPL];
+          if constexpr (CPL == 2) {
+            const float2 t = *reinterpret_cast<const float2*>(Vs + (k + kk) * D + 2 * lane);
+            v[0] = t.x; v[1] = t.y;
+          } else {
+            const float4 t = *reinterpret_cast<const float4*>(Vs + (k + kk) * D + 4 * lane);
+            v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+          }
 #pragma unroll
-          for (int r = 0; r < 4; ++r) {
+          for (int r = 0; r < R; ++r) {
             const float w = kk == 0 ? pv[r].x : kk == 1 ? pv[r].y : kk == 2 ? pv[r].z : pv[r].w;
-            o[r][q][0] = fmaf(w, v.x, o[r][q][0]);
-            o[r][q][1] = fmaf(w, v.y, o[r][q][1]);
-            o[r][q][2] = fmaf(w, v.z, o[r][q][2]);
-            o[r][q][3] = fmaf(w, v.w, o[r][q][3]);
+#pragma unroll
+            for (int q = 0; q < CPL; ++q) o[r][q] = fmaf(w, v[q], o[r][q]);
           }
         }
       }
     }
+#pragma unroll
+    for (int r = 0; r < R; ++r) l[r] = warp_sum(l[r]);
   }
 
   TO* ob = static_cast<TO*>(p.a.out) + size_t(unit) * nt * p.n_q_heads * D;
-  auto store4 = [&](int row, int col, float4 v) {
+  auto store = [&](int row, int col, const auto& v) {  // sizeof(v) / 4 channels
+    constexpr int N = sizeof(v) / 4;
     const int gr = tile * kRows + row;
     TO* dst = ob + (size_t(gr / G) * p.n_q_heads + g * G + gr % G) * D + col;
-    if constexpr (sizeof(TO) == 4) {
-      *reinterpret_cast<float4*>(dst) = v;
-    } else {
-      __align__(8) TO t[4] = {from_f32<TO>(v.x), from_f32<TO>(v.y), from_f32<TO>(v.z), from_f32<TO>(v.w)};
-      *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(t);
-    }
+    __align__(16) TO t[N];
+#pragma unroll
+    for (int e = 0; e < N; ++e) t[e] = from_f32<TO>(v[e]);
+    using Raw = typename std::conditional<sizeof(t) == 16, uint4, typename std::conditional<sizeof(t) == 8, uint2, uint32_t>::type>::type;
+    *reinterpret_cast<Raw*>(dst) = *reinterpret_cast<const Raw*>(t);
   };
   auto store_lse = [&](int row, float mm, float ll) {
     const int gr = tile * kRows + row;
     if (p.a.lse) p.a.lse[(size_t(unit) * p.n_q_heads + g * G + gr % G) * nt + gr / G] = (mm + log2f(ll)) * 0.6931471805599453f;
   };
   if (p.n_splits == 1) {
+    if (warp == kComputeWarps) return;
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int row = ty * 4 + r;
+    for (int r = 0; r < R; ++r) {
+      const int row = warp * R + r;
       if (tile * kRows + row >= n_rows) continue;
       const float inv = l[r] > 0.f ? 1.f / l[r] : 0.f;
+      float v[CPL];
 #pragma unroll
-      for (int q = 0; q < NC; ++q)
-        store4(row, 64 * q + 4 * tx, make_float4(o[r][q][0] * inv, o[r][q][1] * inv, o[r][q][2] * inv, o[r][q][3] * inv));
-      if (tx == 0) store_lse(row, m[r], l[r]);
+      for (int q = 0; q < CPL; ++q) v[q] = o[r][q] * inv;
+      store(row, CPL * lane, v);
+      if (lane == 0) store_lse(row, m[r], l[r]);
     }
     return;
   }
-  // ---- the ranks' partial results: O where Q was, maxima and sums beside it; rank k finishes rows
-  // [32 k / n, 32 (k + 1) / n), adding the ranks in order
-  __syncthreads();
+  // ---- the ranks' partial results: O where Q was (its rows were this warp's alone), maxima and sums beside it; rank k
+  // finishes rows [32 k / n, 32 (k + 1) / n), adding the ranks in order
+  if (warp < kComputeWarps) {
+    __syncwarp();
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < R; ++r) {
+      float* dst = Qs + (warp * R + r) * D + CPL * lane;
 #pragma unroll
-    for (int q = 0; q < NC; ++q)
-      *reinterpret_cast<float4*>(Qs + (ty * 4 + r) * D + 64 * q + 4 * tx) = make_float4(o[r][q][0], o[r][q][1], o[r][q][2], o[r][q][3]);
-    if (tx == 0) { part_m[ty * 4 + r] = m[r]; part_l[ty * 4 + r] = l[r]; }
+      for (int q = 0; q < CPL; ++q) dst[q] = o[r][q];
+      if (lane == 0) { part_m[warp * R + r] = m[r]; part_l[warp * R + r] = l[r]; }
+    }
   }
   __syncwarp();
   cluster_sync_all();
@@ -344,7 +407,8 @@ __global__ void __launch_bounds__(kThreads) attention_simt_kernel(SimtParams p) 
         acc.z = fmaf(w, po[k].z, acc.z); acc.w = fmaf(w, po[k].w, acc.w);
       }
     const float inv = ll > 0.f ? 1.f / ll : 0.f;
-    store4(row, col, make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv));
+    const float v[4] = {acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv};
+    store(row, col, v);
     if (col == 0) store_lse(row, mm, ll);
   }
   __syncwarp();
@@ -389,9 +453,8 @@ int launch_attention_simt(const actqkv_config* cfg, const Batch& b, const AttnAr
   const float scale = cfg->sm_scale > 0.f ? cfg->sm_scale : 1.f / sqrtf(float(cfg->head_dim));
   p.scale_log2 = scale * 1.4426950408889634f;
   const int tiles = (a.n_tokens * p.group + kRows - 1) / kRows;
-  // ranks per key stream: doubled as long as all CTAs are resident at once (shared memory lets an SM
-  // hold four of them at D = 64, two at D = 128)
-  const int64_t slots = int64_t(kNumSMs) * (cfg->head_dim == 64 ? 4 : 2);
+  // ranks per key stream: doubled as long as all CTAs are resident at once (two per SM)
+  const int64_t slots = int64_t(kNumSMs) * 2;
   p.n_splits = 1;
   while (p.n_splits < kMaxSplits && int64_t(tiles) * cfg->n_kv_heads * b.units() * p.n_splits * 2 <= slots) p.n_splits *= 2;
   const dim3 grid(tiles * p.n_splits, cfg->n_kv_heads, b.units());

@@ -81,3 +81,15 @@ def test_general_attention_against_fp64(dtype, D, hq, hkv, units, nt, past, page
             assert err.max().item() < score * V.abs().max().item()
             assert err.mean().item() < 0.01 * score * V.abs().max().item()
             assert (lse[u, g * G:(g + 1) * G].double() - torch.logsumexp(s, -1)).abs().max().item() < score + 1e-6
+
+
+# The keys ahead of the selection (64 initial ones, the local past, the step's own) end on a chunk, one before and one
+# behind it; fewer of them than ranks; several rows per lane group and rows past the last token.
+EARLY_EDGES = [("f32", 64, 4, 2, 1, nt, past, 16, 0) for nt in (63, 64, 65) for past in (704, 705)] + [
+    ("f32", 64, 4, 2, 40, 16, 832, 16, 0), ("f32", 128, 4, 1, 1, 31, 897, 16, 0), ("f32", 128, 4, 1, 1, 32, 768, 16, 0),
+    ("bf16", 64, 8, 2, 1, 127, 761, 16, 8), ("bf16", 128, 2, 1, 2, 33, 831, 16, 0), ("bf16", 64, 2, 2, 1, 1, 704, 16, 0)]
+
+
+@pytest.mark.parametrize("dtype,D,hq,hkv,units,nt,past,page,local", EARLY_EDGES)
+def test_keys_ahead_of_the_selection(dtype, D, hq, hkv, units, nt, past, page, local):
+    test_general_attention_against_fp64(dtype, D, hq, hkv, units, nt, past, page, local)
