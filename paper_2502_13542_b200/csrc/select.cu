@@ -248,12 +248,31 @@ __device__ __forceinline__ int rank_of(uint32_t k, int i, const uint32_t* keys, 
 // phases once before the dependency wait, on 32 made-up scores and without a global access (the rehearsal), and again
 // after it.
 constexpr int kRankMax = 384;
-template <bool kFused, int kKeys>
+
+// The scores of one layer taken inside the selection (D > 0): blocks of 1 KiB, mean aggregation.
+struct ScoreArgs {
+  const float* probe_kv;
+  const void* repr_k;
+  const float* repr_inv_norm;
+  float* scores_out;
+  int r;
+};
+constexpr uint32_t kGroupBytes = 4096;               // four blocks
+constexpr int kScoreKeys = 256;                      // key threads of that form
+constexpr int kScoreMaxCap = 128, kScoreMaxSeqs = 4;
+constexpr int kScoreSlots = kScoreMaxCap / 4 / (kScoreKeys / 32);       // groups of a key warp at most
+constexpr int kScoreSmem = 136 * 1024;               // 1 + 4 + 128.3 KiB at kScoreMaxCap and eight rows a block
+// scores and keys, then the inverse norms, the groups and a barrier for each
+__host__ __device__ inline size_t keys_bytes(int n_cap) { return (size_t(n_cap) + 127) / 128 * 128 * 8; }
+__host__ __device__ inline size_t norms_bytes(int n_cap, int r) { return (size_t(n_cap) * r * 4 + 127) / 128 * 128; }
+__host__ __device__ inline int slots_of(int n_cap) { return (n_cap + 4 * (kScoreKeys / 32) - 1) / (4 * (kScoreKeys / 32)); }
+
+template <bool kFused, int kKeys, typename T, int D>
 __global__ void __launch_bounds__(kKeys + 32)
 select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_cand,
               int32_t* __restrict__ sel_count, int32_t* __restrict__ sel_idx, int n_kv_heads,
-              int n_cap, int cap_blocks, int n_layers, int32_t* status, ChainParams ch) {
-  extern __shared__ uint32_t sel_smem[];       // the head's scores [n_cap] (fp32), then their keys, each padded to a multiple of 128
+              int n_cap, int cap_blocks, int n_layers, int32_t* status, ChainParams ch, ScoreArgs sa) {
+  extern __shared__ __align__(128) uint32_t sel_smem[];       // the head's scores [n_cap] (fp32), then their keys, each padded to a multiple of 128
   constexpr int kWarps = kKeys / 32;
   __shared__ int warp_tot[2][kWarps];
   __shared__ float sh_thetas[2][8];            // the densities of the cluster's heads (written by their CTAs), one set per pass
@@ -275,12 +294,44 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
     asm volatile("barrier.cluster.arrive.release;" ::: "memory");
   }
   grid_launch_dependents();
-  const int n_real = min(n_cand[unit / n_layers], n_cap);
+  const int n_given = n_cand[unit / n_layers], n_real = min(n_given, n_cap);
   const bool ranked = n_real <= min(kRankMax, kKeys);
   const float* s = scores + (size_t(unit) * n_kv_heads + g) * n_cap;
   int32_t* out = sel_idx + (size_t(unit) * n_kv_heads + g) * cap_blocks;
   float* sc = reinterpret_cast<float*>(sel_smem);
   uint32_t* keys = sel_smem + (n_cap + 127) / 128 * 128;
+  // ---- the scores' table: key warp w owns groups w, w + kWarps, ... of four blocks; they and the inverse norms come ahead
+  // of the dependency wait
+  constexpr int VN = 16 / sizeof(T), DD = D > 0 ? D : 128, LPR = DD / VN, RPP = 32 / LPR;
+  const size_t head = size_t(unit) * n_kv_heads + g;
+  unsigned char* after_keys = reinterpret_cast<unsigned char*>(sel_smem) + keys_bytes(n_cap);
+  float* norms = reinterpret_cast<float*>(after_keys);
+  unsigned char* groups = after_keys + norms_bytes(n_cap, sa.r);
+  uint64_t* group_bar = reinterpret_cast<uint64_t*>(groups + size_t(kWarps) * slots_of(n_cap) * kGroupBytes) + warp * kScoreSlots;
+  groups += size_t(warp) * slots_of(n_cap) * kGroupBytes;
+  if constexpr (D > 0) {
+    static_assert(kKeys == kScoreKeys, "the groups are laid out for its warps");
+    if (!control) {
+      if (lane < kScoreSlots) {                      // a lane per group
+        const uint32_t bar = smem(group_bar + lane);
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        const int b = 4 * (warp + lane * kWarps), nb = min(4, n_real - b);
+        if (nb > 0) {
+          const uint32_t bytes = uint32_t(nb) * 1024u;
+          const unsigned char* src = static_cast<const unsigned char*>(sa.repr_k) + (head * n_cap + b) * 1024;
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+          asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                       ::"r"(smem(groups + lane * kGroupBytes)), "l"(src), "r"(bytes), "r"(bar) : "memory");
+        }
+      }
+      __syncwarp();
+      const float* inv = sa.repr_inv_norm + head * n_cap * sa.r;
+      for (int i = tid; i < n_real * sa.r; i += kKeys) norms[i] = __ldg(inv + i);
+    } else if (lane == 0 && g == 0 && n_given > n_cap) {
+      set_status(status, ACTQKV_DEV_NCAND_CLAMPED);
+    }
+  }
 #pragma unroll 1
   for (int pass = 0; pass < 2; ++pass) {
     asm volatile("" : "+r"(pass));             // one body for both passes
@@ -293,6 +344,69 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
     double b_rem = 0.0, rest = 0.0;
     int no_hist = 0;
     if (!control) {
+      if constexpr (D > 0) {
+        float pv[VN], sq = 0.f;
+        const float* pg = sa.probe_kv + head * DD + (lane % LPR) * VN;
+#pragma unroll
+        for (int e = 0; e < VN; e += 4) {
+          const float4 x = real ? __ldg(reinterpret_cast<const float4*>(pg + e)) : make_float4(1.f, 1.f, 1.f, 1.f);
+          pv[e] = x.x; pv[e + 1] = x.y; pv[e + 2] = x.z; pv[e + 3] = x.w;
+        }
+        // the probe's norm: every group of LPR lanes holds the whole probe
+#pragma unroll
+        for (int e = 0; e < VN; ++e) sq = fmaf(pv[e], pv[e], sq);
+#pragma unroll
+        for (int o = LPR >> 1; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        const bool bad = !(sq > 0.f) || !isfinite(sq);
+        if (bad && lane == 0 && 4 * warp < n) set_status(status, ACTQKV_DEV_BAD_PROBE);
+        const float inv_pn = bad ? 0.f : rsqrtf(sq);
+        if (!real) key_sync<kKeys>();            // the norms are written
+        for (int i = 0; 4 * (warp + i * kWarps) < n; ++i) {
+          const int b = 4 * (warp + i * kWarps);
+          bool landed = !real;                   // (the rehearsal does not care what it scores)
+          for (uint32_t k = 0; k < (1u << 20) && !landed; ++k) {        // bounded
+            uint32_t ok;
+            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.b32 %0, 1, 0, p;\n\t}"
+                         : "=r"(ok) : "r"(smem(group_bar + i)), "r"(0u) : "memory");
+            landed = ok != 0;
+          }
+          if (!landed && lane == 0) set_status(status, ACTQKV_DEV_TIMEOUT);     // goes on with whatever arrived
+          __syncwarp();
+          const uint4* rows = reinterpret_cast<const uint4*>(groups + i * kGroupBytes) + lane;
+          float accb[4];
+#pragma unroll
+          for (int bi = 0; bi < 4; ++bi) {
+            accb[bi] = 0.f;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {                      // the block's two vectors
+              const int u = 2 * bi + k, row = b * sa.r + u * RPP + lane / LPR;
+              float x[VN];
+              Vec16<T>::unpack(rows[u * 32], x);
+              float dot = 0.f;
+#pragma unroll
+              for (int e = 0; e < VN; ++e) dot = fmaf(pv[e], x[e], dot);
+              accb[bi] = fmaf(dot, row < n * sa.r ? norms[row] : 0.f, accb[bi]);
+            }
+          }
+          // the four block sums are reduced together: halves swap block pairs, quarters swap blocks, then three steps
+          // inside each quarter
+          const bool up16 = lane & 16, up8 = lane & 8;
+          const float t0 = __shfl_xor_sync(0xffffffffu, up16 ? accb[0] : accb[2], 16);
+          const float t1 = __shfl_xor_sync(0xffffffffu, up16 ? accb[1] : accb[3], 16);
+          const float k0 = (up16 ? accb[2] : accb[0]) + t0, k1 = (up16 ? accb[3] : accb[1]) + t1;
+          float k = (up8 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, up8 ? k0 : k1, 8);
+          k += __shfl_xor_sync(0xffffffffu, k, 4);
+          k += __shfl_xor_sync(0xffffffffu, k, 2);
+          k += __shfl_xor_sync(0xffffffffu, k, 1);
+          const int blk = b + 2 * (lane >> 4) + ((lane >> 3) & 1);
+          if ((lane & 7) == 0 && blk < n) {
+            const float score = k * inv_pn / float(sa.r);
+            sc[blk] = score;
+            if (real) sa.scores_out[head * n_cap + blk] = score;
+          }
+        }
+        key_sync<kKeys>();                       // the scores are complete
+      }
       // the scores are fetched once, by all threads at a time; density and selection read them from here
       float m = -INFINITY;
       for (int i0 = tid; i0 < 4 * n4; i0 += 4 * kKeys) {
@@ -300,13 +414,16 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int i = i0 + u * kKeys;
-          x[u] = i < n ? (real ? s[i] : float(i) * 0.03f) : 0.f;
+          x[u] = i < n ? (D > 0 ? sc[i] : real ? s[i] : float(i) * 0.03f) : 0.f;
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int i = i0 + u * kKeys;
           if (u > 0 && i >= 4 * n4) break;
-          if (kFused && i < n) { sc[i] = x[u]; m = fmaxf(m, ch.beta * x[u]); }
+          if (kFused && i < n) {
+            if (D == 0) sc[i] = x[u];
+            m = fmaxf(m, ch.beta * x[u]);
+          }
           keys[i] = i < n ? score_key(x[u]) : 0u;
         }
       }
@@ -458,9 +575,21 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
   }
 }
 
+// One layer whose scores the selection takes itself: small tables of 1 KiB blocks, which the CTA of a KV head
+// brings into shared memory while the kernel before it runs.  It saves a launch and the hand-over of the scores, and costs
+// a head's products on one SM instead of eight: score and selection of one sequence chained in a graph take 3.7 / 4.4 /
+// 5.8 / 9.1 us at 8 / 40 / 128 / 251 candidates, as two kernels 4.4 / 4.6 / 4.8 / 5.6, with eight sequences 5.1 / 5.7 /
+// 7.4 / 11.7 and 4.8 / 5.4 / 5.6 / 13.1; behind bias + probe, where the copies cost nothing, a window of a prompt is 3 us
+// shorter at up to 62 candidates, 0.3 at 152, and 2.5 longer at 251 (a prompt of 8,103 tokens 898 -> 844 us).
+bool scores_in_selection(const actqkv_config* cfg, const Batch& b) {
+  const size_t block_bytes = size_t(cfg->n_repr) * cfg->head_dim * elt_size(cfg);
+  return b.n_layers == 1 && cfg->n_kv_heads <= 8 && cfg->cap_blocks > 0 && cfg->agg_mode != ACTQKV_AGG_MAX && block_bytes == 1024 &&
+         cfg->n_cap > 0 && cfg->n_cap <= kScoreMaxCap && b.n_seq <= kScoreMaxSeqs;
+}
+
 int launch_cutoff(const actqkv_config* cfg, const Batch& b, const float* scores, const float* theta_in,
                   float* theta_out, const int32_t* n_cand, void* budget_state, int32_t* sel_idx,
-                  int32_t* sel_count, float* budget_real, int32_t* status, cudaStream_t st) {
+                  int32_t* sel_count, float* budget_real, int32_t* status, cudaStream_t st, const ScoreArgs* score_args = nullptr) {
   if (cfg->thetabar_mode == ACTQKV_THETABAR_ALG1 && (b.layer0 != 0 || b.n_layers != cfg->n_layers))
     return ACTQKV_ERR_UNSUPPORTED;
   if (size_t(cfg->n_cap) * 8 > 200 * 1024) return ACTQKV_ERR_SHAPE;
@@ -471,16 +600,28 @@ int launch_cutoff(const actqkv_config* cfg, const Batch& b, const float* scores,
   p.n_kv_heads = cfg->n_kv_heads; p.n_cap = cfg->n_cap; p.L = cfg->n_layers; p.Lb = b.n_layers;
   p.layer0 = b.layer0; p.k_blocks = cfg->k_blocks; p.cap_blocks = cfg->cap_blocks;
   p.thetabar_mode = cfg->thetabar_mode; p.beta = cfg->beta;
-  const size_t sm_sel = (size_t(cfg->n_cap) + 127) / 128 * 128 * 8;        // scores and keys
   const bool fused = b.n_layers == 1 && cfg->n_kv_heads <= 8 && cfg->cap_blocks > 0;
   // 512 key threads where 256 would hold several candidates each and the CTAs have the SMs to themselves; a grid that fills
   // the SMs keeps the narrow form, which becomes resident beside two CTAs of the streaming scores (288 threads x 56
   // registers; 16 sequences of 32k-131k tokens, a decode step of two layers: 168 us).
   const bool wide = cfg->n_cap > 256 && b.units() * cfg->n_kv_heads <= kNumSMs / 2;
-  auto kern = fused ? (wide ? select_kernel<true, 512> : select_kernel<true, 256>)
-                    : (wide ? select_kernel<false, 512> : select_kernel<false, 256>);
+  using bf16 = __nv_bfloat16;
+  auto kern = fused ? (wide ? select_kernel<true, 512, float, 0> : select_kernel<true, 256, float, 0>)
+                    : (wide ? select_kernel<false, 512, float, 0> : select_kernel<false, 256, float, 0>);
+  ScoreArgs sa = {};
+  size_t sm_sel = keys_bytes(cfg->n_cap);
+  if (score_args) {
+    sa = *score_args;
+    const bool half = cfg->dtype == ACTQKV_BF16;
+    kern = cfg->head_dim == 128 ? (half ? select_kernel<true, kScoreKeys, bf16, 128> : select_kernel<true, kScoreKeys, float, 128>)
+                                : (half ? select_kernel<true, kScoreKeys, bf16, 64> : select_kernel<true, kScoreKeys, float, 64>);
+    sm_sel += norms_bytes(cfg->n_cap, sa.r) + size_t(kScoreKeys / 32) * (slots_of(cfg->n_cap) * kGroupBytes + kScoreSlots * 8);
+  }
+  static std::atomic<bool> carved[8][kMaxDevices], opted_in[8][kMaxDevices];
+  const int form = score_args ? 4 + 2 * (cfg->head_dim == 128) + (cfg->dtype == ACTQKV_BF16) : 2 * wide + fused;
   if (sm_sel > 40 * 1024 &&
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm_sel)) != cudaSuccess)
+      !(score_args ? opt_in_shared_memory(kern, kScoreSmem, opted_in[form])
+                   : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm_sel)) == cudaSuccess))
     return ACTQKV_ERR_LAUNCH;
   if (!fused) {
     const size_t sm_chain = sizeof(float) * ((size_t(b.n_layers) * cfg->n_kv_heads + 1) & ~size_t(1)) +
@@ -506,8 +647,7 @@ int launch_cutoff(const actqkv_config* cfg, const Batch& b, const float* scores,
     if (cudaLaunchKernelEx(&lcc, cutoff_chain_kernel, p) != cudaSuccess) return ACTQKV_ERR_LAUNCH;
     if (cfg->cap_blocks == 0) return ACTQKV_OK;
   }
-  static std::atomic<bool> carved[4][kMaxDevices];
-  prefer_max_shared(kern, carved[2 * wide + fused]);
+  prefer_max_shared(kern, carved[form]);
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3(cfg->n_kv_heads, b.units(), 1);
   lc.blockDim = dim3((wide ? 512 : 256) + 32, 1, 1);
@@ -522,7 +662,7 @@ int launch_cutoff(const actqkv_config* cfg, const Batch& b, const float* scores,
   lc.attrs = attr;
   lc.numAttrs = 2;                  // every kernel of the chain waits for its predecessor before it reads
   if (cudaLaunchKernelEx(&lc, kern, scores, n_cand, sel_count, sel_idx, cfg->n_kv_heads, cfg->n_cap,
-                         cfg->cap_blocks, b.n_layers, status, p) != cudaSuccess)
+                         cfg->cap_blocks, b.n_layers, status, p, sa) != cudaSuccess)
     return ACTQKV_ERR_LAUNCH;
   return launch_status();
 }
@@ -557,6 +697,10 @@ extern "C" int actqkv_score_select(const actqkv_config* cfg, const actqkv_batch*
   ACTQKV_REQUIRE_PTR(sel_idx);
   if (!n_cand || !budget_state || !sel_count) return ACTQKV_ERR_NULL;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (scores_in_selection(cfg, b)) {
+    const ScoreArgs sa = {probe_kv, repr_k, repr_inv_norm, scores, cfg->n_repr};
+    return launch_cutoff(cfg, b, scores, nullptr, theta, n_cand, budget_state, sel_idx, sel_count, budget_real, status, st, &sa);
+  }
   rc = launch_scores(cfg, b, probe_kv, repr_k, repr_inv_norm, n_cand, scores, status, st);
   if (rc) return rc;
   return launch_cutoff(cfg, b, scores, nullptr, theta, n_cand, budget_state, sel_idx, sel_count,

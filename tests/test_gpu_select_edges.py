@@ -81,3 +81,45 @@ def test_density_and_selection_of_one_layer(seqs, n):
             assert 1 <= k <= min(c, m)
             for g in range(8):
                 assert sel[u, g].tolist() == pick(scores[u, g, :m].tolist(), k) + [-1] * (c - k)
+
+
+@pytest.mark.parametrize("dtype,D,r", [("bf16", 128, 4), ("bf16", 64, 8), ("f32", 128, 2), ("f32", 64, 4)])
+@pytest.mark.parametrize("n", [0, 1, 3, 31, 32, 33, 65, 127, 128, 129])
+def test_scores_taken_by_the_selection(dtype, D, r, n):
+    """Small tables of 1 KiB blocks (up to 128 candidates, 4 sequences): the bits of the two-kernel form, which five
+    sequences take, and the same sets; a count beyond the table and a probe of zeros are reported."""
+    import torch
+    from paper_2502_13542_b200 import binding as B
+    L, c = 2, 7
+    spec = wl.llama3_8b_layer().replace(n_layers=L, k_blocks=c, cap_blocks=c, n_kv_heads=8, head_dim=D, dtype=dtype, n_repr=r)
+    cap = max(n, 1)
+    cfg = B.make_config(spec, n_cap=cap, beta=4.0)
+    gen = torch.Generator(device="cuda").manual_seed(n + D)
+    table = torch.randn(5, 8, cap, r, D, device="cuda", generator=gen).to(cfg.torch_dtype)
+    norms = 1.0 / table.float().norm(dim=-1)
+    probe = torch.randn(5, 8, D, device="cuda", generator=gen)
+    counts = torch.tensor([n, max(0, n - 1), n // 2, n, n], dtype=torch.int32, device="cuda")
+
+    def run(seqs, probe=probe, counts=counts):
+        out = dict(scores=torch.zeros(seqs, 8, cap, device="cuda"), theta=torch.zeros(seqs, 8, device="cuda"),
+                   sel=torch.full((seqs, 8, c), -7, dtype=torch.int32, device="cuda"),
+                   cnt=torch.zeros(seqs, dtype=torch.int32, device="cuda"),
+                   state=torch.zeros(seqs, 1 + 2 * L, dtype=torch.float64, device="cuda"))
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        for layer in range(L):
+            B.score_select(cfg, B.Batch(seqs, 1, layer), probe[:seqs].contiguous(), table[:seqs].contiguous(),
+                           norms[:seqs].contiguous(), counts[:seqs].contiguous(), out["state"], out["scores"], out["theta"],
+                           out["sel"], out["cnt"], None, status)
+        torch.cuda.synchronize()
+        return out, int(status.item())
+
+    (small, bits), (both, _) = run(4), run(5)
+    assert bits == 0
+    for key, x in small.items():
+        assert torch.equal(x, both[key][:4]), key
+    zero = probe.clone()
+    zero[1, 2] = 0
+    want, got = run(5, zero, counts + 1 - counts.clamp(max=0)), run(4, zero, counts + 1 - counts.clamp(max=0))
+    assert want[1] == got[1] != 0
+    for key, x in got[0].items():
+        assert torch.equal(x, want[0][key][:4]), key
