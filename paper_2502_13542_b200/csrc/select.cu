@@ -6,13 +6,13 @@
 //                        the layers shallow -> deep in fp64: B^l from Eq. 12, the granted
 //                        integer c^l, the running B_kv and the density history.
 //   select_kernel        one CTA per (unit, KV head).  Scores become order-preserving 32-bit
-//                        keys in shared memory; a binary search on the bits finds the c-th
-//                        largest key; equal keys are admitted lowest index first; the survivors
-//                        are compacted in ascending block order with block-wide scans.
+//                        keys in shared memory; up to 384 keys are ranked against one another, of more the
+//                        c-th largest is found by a search on the bits; equal keys are admitted lowest index
+//                        first; the survivors are compacted in ascending block order.
 // A call for one layer (the usual layer-by-layer use) runs select_kernel alone: the Hkv CTAs of a
 // sequence form a thread-block cluster, each takes its head's density, they exchange the values
 // through distributed shared memory, every CTA evaluates Eq. 12 for itself and the first one
-// writes the budget state back.
+// writes the budget state back.  Where the table is small it takes the scores, too.
 #include "common.cuh"
 #include "stages.cuh"
 
