@@ -143,7 +143,9 @@ typedef struct actqkv_config {
   /* Test hooks of the failure-detection path (leave both 0).  With test_wait_limit > 0 the decode
    * attention kernel gives its device-side waits that many polls instead of its normal limit and
    * never issues the K copy of tile test_drop_k_tile of each CTA, so that the wait for that tile runs
-   * out: the kernel must set ACTQKV_DEV_TIMEOUT, return, and leave the context usable. */
+   * out: the kernel must set ACTQKV_DEV_TIMEOUT, return, and leave the context usable.  The selection of one
+   * layer takes the same limit; the CTA of KV head test_drop_k_tile never hands out its density, and with
+   * n_kv_heads + g that of head g never fetches its first four blocks where it takes the scores itself. */
   int32_t test_wait_limit;
   int32_t test_drop_k_tile;
 } actqkv_config;

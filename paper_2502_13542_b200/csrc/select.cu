@@ -32,6 +32,8 @@ struct ChainParams {
   float* budget_real;
   int n_kv_heads, n_cap, L, Lb, layer0, k_blocks, cap_blocks, thetabar_mode;
   float beta;
+  uint32_t polls;          // bound of a device-side wait
+  int drop;                // test hook: what select_kernel never sends (-1: nothing)
 };
 
 // Eq. 12 for one layer with n > 0 candidates: returns the granted count c and the un-rounded
@@ -228,6 +230,17 @@ __device__ __forceinline__ int rank_of(uint32_t k, int i, const uint32_t* keys, 
   return r + __popc(same & ((1u << (i & 31)) - 1u));
 }
 
+// Waits (bounded) for phase 0 of an mbarrier.
+__device__ __forceinline__ bool wait_phase0(uint32_t bar, uint32_t polls) {
+  for (uint32_t i = 0; i < polls; ++i) {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\tselp.b32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(bar) : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+
 // kFused: the call holds one layer; the grid is launched as clusters of n_kv_heads CTAs (one
 // sequence each) and the cut-off chain of that layer is evaluated here (ch), else sel_count is
 // an input written by cutoff_chain_kernel.
@@ -278,13 +291,14 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
   __shared__ float sh_thetas[2][8];            // the densities of the cluster's heads (written by their CTAs), one set per pass
   __shared__ __align__(8) uint64_t sh_bar[2];  // a pass's densities have arrived
   __shared__ float red_m[kWarps], red_z[kWarps], red_e[kWarps];
-  __shared__ int sh_count;
+  __shared__ int sh_count, sh_late;            // the granted count; a wait ran out
   const int g = blockIdx.x, unit = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool control = warp == kWarps;
   auto smem = [](const void* x) { return uint32_t(__cvta_generic_to_shared(x)); };
   // A peer's shared memory may be written only once that peer runs: every CTA says so here, and waits for
   // the others just ahead of its first remote store.
   if constexpr (kFused) {
+    if (tid == 0) sh_late = 0;
     if (control && lane < 2) {
       const uint32_t bytes = 4u * uint32_t(n_kv_heads), bar = smem(sh_bar + lane);
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
@@ -317,7 +331,7 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         const int b = 4 * (warp + lane * kWarps), nb = min(4, n_real - b);
-        if (nb > 0) {
+        if (nb > 0 && !(b == 0 && ch.drop == n_kv_heads + g)) {
           const uint32_t bytes = uint32_t(nb) * 1024u;
           const unsigned char* src = static_cast<const unsigned char*>(sa.repr_k) + (head * n_cap + b) * 1024;
           asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
@@ -363,14 +377,9 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
         if (!real) key_sync<kKeys>();            // the norms are written
         for (int i = 0; 4 * (warp + i * kWarps) < n; ++i) {
           const int b = 4 * (warp + i * kWarps);
-          bool landed = !real;                   // (the rehearsal does not care what it scores)
-          for (uint32_t k = 0; k < (1u << 20) && !landed; ++k) {        // bounded
-            uint32_t ok;
-            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.b32 %0, 1, 0, p;\n\t}"
-                         : "=r"(ok) : "r"(smem(group_bar + i)), "r"(0u) : "memory");
-            landed = ok != 0;
+          if (real && !wait_phase0(smem(group_bar + i), ch.polls)) {            // goes on with whatever arrived
+            if (lane == 0) { sh_late = 1; set_status(status, ACTQKV_DEV_TIMEOUT); }
           }
-          if (!landed && lane == 0) set_status(status, ACTQKV_DEV_TIMEOUT);     // goes on with whatever arrived
           __syncwarp();
           const uint4* rows = reinterpret_cast<const uint4*>(groups + i * kGroupBytes) + lane;
           float accb[4];
@@ -474,21 +483,14 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
         if (lane == 0 && !ch.theta_in && ch.theta_out && real) ch.theta_out[uh] = th_own;
       }
       const uint32_t bar = smem(sh_bar + pass);
-      if (lane < n_kv_heads) {
+      if (lane < n_kv_heads && !(real && ch.drop == g)) {
         uint32_t dst, far;
         asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(smem(&sh_thetas[pass][g])), "r"(lane));
         asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(far) : "r"(bar), "r"(lane));
         asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
                      ::"r"(dst), "r"(__float_as_uint(th_own)), "r"(far) : "memory");
       }
-      bool here = false;
-      for (uint32_t i = 0; i < (1u << 20) && !here; ++i) {        // bounded
-        uint32_t ok;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\tselp.b32 %0, 1, 0, p;\n\t}"
-                     : "=r"(ok) : "r"(bar) : "memory");
-        here = ok != 0;
-      }
-      if (!here && lane == 0) set_status(status, ACTQKV_DEV_TIMEOUT);
+      if (!wait_phase0(bar, ch.polls) && lane == 0) { sh_late = 1; set_status(status, ACTQKV_DEV_TIMEOUT); }
       double sum = 0.0;
       for (int h = 0; h < n_kv_heads; ++h) sum += double(sh_thetas[pass][h]);
       const double th = sum / double(n_kv_heads);
@@ -573,6 +575,18 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
     }
     __syncthreads();                             // the next pass writes what this one reads
   }
+  // A CTA whose wait ran out may not leave before what is still on its way to its shared memory has arrived: its own
+  // copies, and the densities of peers that are late (they have sent theirs once they are at this barrier or have exited,
+  // which counts as arriving).  Where all densities arrived no peer has anything left to send.
+  if constexpr (kFused) {
+    if (sh_late) {
+      if constexpr (D > 0)
+        for (int i = 0; !control && 4 * (warp + i * kWarps) < n_real; ++i) wait_phase0(smem(group_bar + i), ch.polls);
+      asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+      wait_phase0(smem(sh_bar), ch.polls);
+      wait_phase0(smem(sh_bar + 1), ch.polls);
+    }
+  }
 }
 
 // One layer whose scores the selection takes itself: small tables of 1 KiB blocks, which the CTA of a KV head
@@ -600,6 +614,8 @@ int launch_cutoff(const actqkv_config* cfg, const Batch& b, const float* scores,
   p.n_kv_heads = cfg->n_kv_heads; p.n_cap = cfg->n_cap; p.L = cfg->n_layers; p.Lb = b.n_layers;
   p.layer0 = b.layer0; p.k_blocks = cfg->k_blocks; p.cap_blocks = cfg->cap_blocks;
   p.thetabar_mode = cfg->thetabar_mode; p.beta = cfg->beta;
+  p.polls = cfg->test_wait_limit > 0 ? uint32_t(cfg->test_wait_limit) : 1u << 20;
+  p.drop = cfg->test_wait_limit > 0 ? cfg->test_drop_k_tile : -1;
   const bool fused = b.n_layers == 1 && cfg->n_kv_heads <= 8 && cfg->cap_blocks > 0;
   // 512 key threads where 256 would hold several candidates each and the CTAs have the SMs to themselves; a grid that fills
   // the SMs keeps the narrow form, which becomes resident beside two CTAs of the streaming scores (288 threads x 56

@@ -86,3 +86,41 @@ def test_what_a_rank_that_gave_up_leaves_behind_does_not_reach_the_output(nt, sp
         torch.cuda.synchronize()
         assert int(st.status.item()) & B.DEV_TIMEOUT
         assert torch.isfinite(out).all()
+
+
+@pytest.mark.parametrize("seqs,n,dropped", [(1, 100, 0), (1, 100, 7), (4, 128, 9), (2, 5, 8), (1, 300, 3), (12, 300, 5), (1, 129, 11)])
+def test_selection_whose_heads_or_rows_are_late_ends_with_the_timeout_bit(seqs, n, dropped):
+    """One KV head's CTA never hands out its density (dropped < 8), or never fetches its first rows (8 + head) and is late with
+    it (tables of more than 128 candidates, or five sequences, are not fetched: nothing is late there).  CTAs that gave up stay
+    until their peers can no longer write to them; the status says so, and the next call gives the bits of the first."""
+    import torch
+    from paper_2502_13542_b200 import binding as B
+    spec = wl.llama3_8b_layer().replace(n_layers=1, k_blocks=5, cap_blocks=5)
+    cfg = B.make_config(spec, n_cap=n)
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    table = torch.randn(seqs, 8, n, 4, 128, device="cuda", generator=gen).bfloat16()
+    norms = 1.0 / table.float().norm(dim=-1)
+    probe = torch.randn(seqs, 8, 128, device="cuda", generator=gen)
+    n_cand = torch.full((seqs,), n, dtype=torch.int32, device="cuda")
+
+    def run(c):
+        out = dict(scores=torch.zeros(seqs, 8, n, device="cuda"), theta=torch.zeros(seqs, 8, device="cuda"),
+                   sel=torch.zeros(seqs, 8, 5, dtype=torch.int32, device="cuda"), cnt=torch.zeros(seqs, dtype=torch.int32, device="cuda"))
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        state = torch.zeros(seqs, 3, dtype=torch.float64, device="cuda")
+        B.score_select(c, B.Batch(seqs, 1, 0), probe, table, norms, n_cand, state, out["scores"], out["theta"], out["sel"],
+                       out["cnt"], None, status)
+        torch.cuda.synchronize()                      # returns: no CTA hung
+        return out, int(status.item())
+
+    good, s = run(cfg)
+    assert s == 0
+    broken = B.make_config(spec, n_cap=n)
+    broken.test_wait_limit, broken.test_drop_k_tile = 2000, dropped
+    for _ in range(3):
+        _, s = run(broken)
+        assert s == (B.DEV_TIMEOUT if dropped < 8 or (n <= 128 and seqs <= 4) else 0)
+        again, s = run(cfg)
+        assert s == 0
+        for key, x in good.items():
+            assert torch.equal(x, again[key]), key
