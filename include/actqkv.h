@@ -145,7 +145,8 @@ typedef struct actqkv_config {
    * never issues the K copy of tile test_drop_k_tile of each CTA, so that the wait for that tile runs
    * out: the kernel must set ACTQKV_DEV_TIMEOUT, return, and leave the context usable.  The selection of one
    * layer takes the same limit; the CTA of KV head test_drop_k_tile never hands out its density, and with
-   * n_kv_heads + g that of head g never fetches its first four blocks where it takes the scores itself. */
+   * n_kv_heads + g that of head g never fetches its first four blocks where it takes the scores itself
+   * (actqkv_step). */
   int32_t test_wait_limit;
   int32_t test_drop_k_tile;
 } actqkv_config;

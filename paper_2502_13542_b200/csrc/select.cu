@@ -272,7 +272,7 @@ struct ScoreArgs {
 };
 constexpr uint32_t kGroupBytes = 4096;               // four blocks
 constexpr int kScoreKeys = 256;                      // key threads of that form
-constexpr int kScoreMaxCap = 128, kScoreMaxSeqs = 4;
+constexpr int kScoreMaxCap = 128, kScoreMaxHeads = 16;
 constexpr int kScoreSlots = kScoreMaxCap / 4 / (kScoreKeys / 32);       // groups of a key warp at most
 constexpr int kScoreSmem = 136 * 1024;               // 1 + 4 + 128.3 KiB at kScoreMaxCap and eight rows a block
 // scores and keys, then the inverse norms, the groups and a barrier for each
@@ -590,15 +590,19 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
 }
 
 // One layer whose scores the selection takes itself: small tables of 1 KiB blocks, which the CTA of a KV head
-// brings into shared memory while the kernel before it runs.  It saves a launch and the hand-over of the scores, and costs
-// a head's products on one SM instead of eight: score and selection of one sequence chained in a graph take 3.7 / 4.4 /
-// 5.8 / 9.1 us at 8 / 40 / 128 / 251 candidates, as two kernels 4.4 / 4.6 / 4.8 / 5.6, with eight sequences 5.1 / 5.7 /
-// 7.4 / 11.7 and 4.8 / 5.4 / 5.6 / 13.1; behind bias + probe, where the copies cost nothing, a window of a prompt is 3 us
-// shorter at up to 62 candidates, 0.3 at 152, and 2.5 longer at 251 (a prompt of 8,103 tokens 898 -> 844 us).
+// brings into shared memory while bias + probe of the window runs.  It saves a launch and the hand-over of the scores, and
+// costs a head's products on one SM instead of eight.  Steps of 2 to 512 tokens in tables of 104 rows, one kernel against two, us
+// a layer at 4 / 40 / 96 candidates: one sequence of 8 KV heads -0.7 to -1.8 / -0.3 to -1.1 / -0.1 to -4.1, two -2.2 to +0.9 / -2.2 to
+// +1.0 / -2.1 to +0.5 (the losses at 64 and 128 tokens), three -2.9 to +0.5 / -2.4 to +3.3 / -3.1 to +5.5, four +0.7 to +2.0 / +1.0 to +4.0 /
+// -0.6 to +2.2; 2 KV heads (fp32) gain up to four sequences.  So it is taken up to 16 heads in all.  At 120 candidates of a table
+// of 128 it is even (-2 to +2.9), but a prompt comes through all the smaller counts first.
+// Behind anything shorter than bias + probe the copies are exposed (the append of the step before lets nothing start
+// early): a decode step with attention and append takes 14.6 / 17.9 / 18.5 us as two kernels and 15.2 / 19.4 / 20.6 as one at
+// 8 / 40 / 96 candidates, 27.5 and 29.3 with four sequences at 96, a drafted step of 5 tokens 21.0 and 23.9.
 bool scores_in_selection(const actqkv_config* cfg, const Batch& b) {
   const size_t block_bytes = size_t(cfg->n_repr) * cfg->head_dim * elt_size(cfg);
   return b.n_layers == 1 && cfg->n_kv_heads <= 8 && cfg->cap_blocks > 0 && cfg->agg_mode != ACTQKV_AGG_MAX && block_bytes == 1024 &&
-         cfg->n_cap > 0 && cfg->n_cap <= kScoreMaxCap && b.n_seq <= kScoreMaxSeqs;
+         cfg->n_cap > 0 && cfg->n_cap <= kScoreMaxCap && b.n_seq * cfg->n_kv_heads <= kScoreMaxHeads;
 }
 
 int launch_cutoff(const actqkv_config* cfg, const Batch& b, const float* scores, const float* theta_in,
@@ -699,10 +703,10 @@ extern "C" int actqkv_select_cutoff(const actqkv_config* cfg, const actqkv_batch
                        budget_real, status, reinterpret_cast<cudaStream_t>(stream));
 }
 
-extern "C" int actqkv_score_select(const actqkv_config* cfg, const actqkv_batch* batch, const float* probe_kv,
-                                   const void* repr_k, const float* repr_inv_norm, const int32_t* n_cand,
-                                   void* budget_state, float* scores, float* theta, int32_t* sel_idx,
-                                   int32_t* sel_count, float* budget_real, int32_t* status, void* stream) {
+int actqkv::score_select(const actqkv_config* cfg, const actqkv_batch* batch, const float* probe_kv, const void* repr_k,
+                         const float* repr_inv_norm, const int32_t* n_cand, void* budget_state, float* scores, float* theta,
+                         int32_t* sel_idx, int32_t* sel_count, float* budget_real, int32_t* status, bool behind_probe,
+                         cudaStream_t st) {
   const Batch b = get_batch(batch);
   int rc = check_config(cfg, b);
   if (rc) return rc;
@@ -712,13 +716,19 @@ extern "C" int actqkv_score_select(const actqkv_config* cfg, const actqkv_batch*
   ACTQKV_REQUIRE_PTR(scores);
   ACTQKV_REQUIRE_PTR(sel_idx);
   if (!n_cand || !budget_state || !sel_count) return ACTQKV_ERR_NULL;
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (scores_in_selection(cfg, b)) {
+  if (behind_probe && scores_in_selection(cfg, b)) {
     const ScoreArgs sa = {probe_kv, repr_k, repr_inv_norm, scores, cfg->n_repr};
     return launch_cutoff(cfg, b, scores, nullptr, theta, n_cand, budget_state, sel_idx, sel_count, budget_real, status, st, &sa);
   }
   rc = launch_scores(cfg, b, probe_kv, repr_k, repr_inv_norm, n_cand, scores, status, st);
   if (rc) return rc;
-  return launch_cutoff(cfg, b, scores, nullptr, theta, n_cand, budget_state, sel_idx, sel_count,
-                       budget_real, status, st);
+  return launch_cutoff(cfg, b, scores, nullptr, theta, n_cand, budget_state, sel_idx, sel_count, budget_real, status, st);
+}
+
+extern "C" int actqkv_score_select(const actqkv_config* cfg, const actqkv_batch* batch, const float* probe_kv,
+                                   const void* repr_k, const float* repr_inv_norm, const int32_t* n_cand,
+                                   void* budget_state, float* scores, float* theta, int32_t* sel_idx,
+                                   int32_t* sel_count, float* budget_real, int32_t* status, void* stream) {
+  return score_select(cfg, batch, probe_kv, repr_k, repr_inv_norm, n_cand, budget_state, scores, theta, sel_idx, sel_count,
+                      budget_real, status, false, reinterpret_cast<cudaStream_t>(stream));
 }

@@ -67,6 +67,12 @@ int launch_scores(const actqkv_config* cfg, const Batch& b, const float* probe_k
                   const float* repr_inv_norm, const int32_t* n_cand, float* scores, int32_t* status,
                   cudaStream_t st);
 
+// actqkv_score_select; behind_probe: the stream's kernel before it is bias + probe of a window, long enough for the
+// selection to bring a small table in beside it.
+int score_select(const actqkv_config* cfg, const actqkv_batch* batch, const float* probe_kv, const void* repr_k,
+                 const float* repr_inv_norm, const int32_t* n_cand, void* budget_state, float* scores, float* theta,
+                 int32_t* sel_idx, int32_t* sel_count, float* budget_real, int32_t* status, bool behind_probe, cudaStream_t st);
+
 // Eq. 11 for every (unit, KV head), one CTA each.
 int launch_entropy(const actqkv_config* cfg, const Batch& b, const float* scores, const int32_t* n_cand,
                    float* theta, cudaStream_t st);

@@ -88,11 +88,10 @@ def test_what_a_rank_that_gave_up_leaves_behind_does_not_reach_the_output(nt, sp
         assert torch.isfinite(out).all()
 
 
-@pytest.mark.parametrize("seqs,n,dropped", [(1, 100, 0), (1, 100, 7), (4, 128, 9), (2, 5, 8), (1, 300, 3), (12, 300, 5), (1, 129, 11)])
-def test_selection_whose_heads_or_rows_are_late_ends_with_the_timeout_bit(seqs, n, dropped):
-    """One KV head's CTA never hands out its density (dropped < 8), or never fetches its first rows (8 + head) and is late with
-    it (tables of more than 128 candidates, or five sequences, are not fetched: nothing is late there).  CTAs that gave up stay
-    until their peers can no longer write to them; the status says so, and the next call gives the bits of the first."""
+@pytest.mark.parametrize("seqs,n,dropped", [(1, 100, 0), (1, 100, 7), (2, 5, 4), (1, 300, 3), (12, 300, 5), (1, 600, 6)])
+def test_selection_without_a_head_s_density_ends_with_the_timeout_bit(seqs, n, dropped):
+    """One KV head's CTA never hands out its density.  CTAs that gave up stay until their peers can no longer write to them;
+    the status says so, and the next call gives the bits of the first.  (Rows that are late: test_gpu_select_edges.py.)"""
     import torch
     from paper_2502_13542_b200 import binding as B
     spec = wl.llama3_8b_layer().replace(n_layers=1, k_blocks=5, cap_blocks=5)
@@ -119,7 +118,7 @@ def test_selection_whose_heads_or_rows_are_late_ends_with_the_timeout_bit(seqs, 
     broken.test_wait_limit, broken.test_drop_k_tile = 2000, dropped
     for _ in range(3):
         _, s = run(broken)
-        assert s == (B.DEV_TIMEOUT if dropped < 8 or (n <= 128 and seqs <= 4) else 0)
+        assert s == B.DEV_TIMEOUT
         again, s = run(cfg)
         assert s == 0
         for key, x in good.items():

@@ -86,40 +86,58 @@ def test_density_and_selection_of_one_layer(seqs, n):
 @pytest.mark.parametrize("dtype,D,r", [("bf16", 128, 4), ("bf16", 64, 8), ("f32", 128, 2), ("f32", 64, 4)])
 @pytest.mark.parametrize("n", [0, 1, 3, 31, 32, 33, 65, 127, 128, 129])
 def test_scores_taken_by_the_selection(dtype, D, r, n):
-    """Small tables of 1 KiB blocks (up to 128 candidates, 4 sequences): the bits of the two-kernel form, which five
-    sequences take, and the same sets; a count beyond the table and a probe of zeros are reported."""
+    """Small tables of 1 KiB blocks: a step that takes its probe from its own window (up to 128 candidates and 16 heads) has
+    the scores taken by the selection; the bits are those of score_select, which takes two kernels.  (At 129 rows both do.)"""
     import torch
     from paper_2502_13542_b200 import binding as B
-    L, c = 2, 7
-    spec = wl.llama3_8b_layer().replace(n_layers=L, k_blocks=c, cap_blocks=c, n_kv_heads=8, head_dim=D, dtype=dtype, n_repr=r)
+    L, c, nt, seqs = 2, 7, 3, 2
+    spec = wl.llama3_8b_layer().replace(n_layers=L, k_blocks=c, cap_blocks=c, n_q_heads=8, n_kv_heads=8, head_dim=D, dtype=dtype,
+                                        n_repr=r, window=16)
     cap = max(n, 1)
-    cfg = B.make_config(spec, n_cap=cap, beta=4.0)
+    kw = dict(n_cap=cap, beta=4.0, max_pages=2, n_phys_pages=2)
+    cfg = B.make_config(spec, **kw)
     gen = torch.Generator(device="cuda").manual_seed(n + D)
-    table = torch.randn(5, 8, cap, r, D, device="cuda", generator=gen).to(cfg.torch_dtype)
+    rnd = lambda *shape: torch.randn(*shape, device="cuda", generator=gen)      # noqa: E731
+    table = rnd(seqs, 8, cap, r, D).to(cfg.torch_dtype)
     norms = 1.0 / table.float().norm(dim=-1)
-    probe = torch.randn(5, 8, D, device="cuda", generator=gen)
-    counts = torch.tensor([n, max(0, n - 1), n // 2, n, n], dtype=torch.int32, device="cuda")
+    q = rnd(seqs, nt, 8, D).to(cfg.torch_dtype)
+    kv = torch.zeros_like(q)
+    out = torch.empty_like(q)
 
-    def run(seqs, probe=probe, counts=counts):
-        out = dict(scores=torch.zeros(seqs, 8, cap, device="cuda"), theta=torch.zeros(seqs, 8, device="cuda"),
-                   sel=torch.full((seqs, 8, c), -7, dtype=torch.int32, device="cuda"),
-                   cnt=torch.zeros(seqs, dtype=torch.int32, device="cuda"),
-                   state=torch.zeros(seqs, 1 + 2 * L, dtype=torch.float64, device="cuda"))
-        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    def run(counts, q=q, cfg=cfg):
+        """The step of two layers, and score_select on the probes it left; results and status bits of both."""
+        got, want, bits = [], [], [0, 0]
+        state = torch.zeros(seqs, 1 + 2 * L, dtype=torch.float64, device="cuda")
+        other = state.clone()
         for layer in range(L):
-            B.score_select(cfg, B.Batch(seqs, 1, layer), probe[:seqs].contiguous(), table[:seqs].contiguous(),
-                           norms[:seqs].contiguous(), counts[:seqs].contiguous(), out["state"], out["scores"], out["theta"],
-                           out["sel"], out["cnt"], None, status)
-        torch.cuda.synchronize()
-        return out, int(status.item())
+            st = B.RetrievalState(cfg, n_seq=seqs, n_layers=1, layer0=layer)
+            st.repr_k.copy_(table), st.repr_inv_norm.copy_(norms)
+            st.budget_state, st.n_cand = state, torch.tensor(counts, dtype=torch.int32, device="cuda")
+            st.step(q, kv, kv, out, advance=False)        # (position 0: the attention and the append see none of this)
+            torch.cuda.synchronize()
+            bits[0] |= int(st.status.item()) & ~B.DEV_BAD_SELECTION        # (the attention knows of no candidates)
+            got += [st.scores.clone(), st.theta.clone(), st.sel_idx.clone(), st.sel_count.clone(), state.clone()]
+            st.status.zero_(), st.scores.zero_(), st.theta.zero_(), st.sel_idx.fill_(-7), st.sel_count.zero_()
+            B.score_select(cfg, st.batch, st.probe_kv, st.repr_k, st.repr_inv_norm, st.n_cand, other, st.scores, st.theta,
+                           st.sel_idx, st.sel_count, None, st.status)
+            torch.cuda.synchronize()
+            bits[1] |= int(st.status.item())
+            want += [st.scores, st.theta, st.sel_idx, st.sel_count, other.clone()]
+        for i, (a, b) in enumerate(zip(got, want)):
+            assert torch.equal(a, b), i
+        return bits
 
-    (small, bits), (both, _) = run(4), run(5)
-    assert bits == 0
-    for key, x in small.items():
-        assert torch.equal(x, both[key][:4]), key
-    zero = probe.clone()
-    zero[1, 2] = 0
-    want, got = run(5, zero, counts + 1 - counts.clamp(max=0)), run(4, zero, counts + 1 - counts.clamp(max=0))
-    assert want[1] == got[1] != 0
-    for key, x in got[0].items():
-        assert torch.equal(x, want[0][key][:4]), key
+    assert run([n, n // 2]) == [0, 0]
+    assert run([n, cap + 1]) == [B.DEV_NCAND_CLAMPED] * 2
+    zero = q.clone()
+    zero[1, :, 2] = 0
+    assert run([n, n], q=zero) == [B.DEV_BAD_PROBE if n else 0] * 2
+    if 0 < n <= 128:                                      # the step takes the form in question: only there rows can be late
+        for late, bit in ((99, 0), (8, B.DEV_TIMEOUT), (99, 0)):
+            hooked = B.make_config(spec, **kw)
+            hooked.test_wait_limit, hooked.test_drop_k_tile = 20000, late
+            st = B.RetrievalState(hooked, n_seq=seqs)
+            st.repr_k.copy_(table), st.repr_inv_norm.copy_(norms), st.n_cand.fill_(n)
+            st.step(q, kv, kv, out, advance=False)
+            torch.cuda.synchronize()
+            assert int(st.status.item()) & B.DEV_TIMEOUT == bit
