@@ -275,6 +275,7 @@ constexpr int kScoreKeys = 256;                      // key threads of that form
 constexpr int kScoreMaxCap = 128, kScoreMaxHeads = 16;
 constexpr int kScoreSlots = kScoreMaxCap / 4 / (kScoreKeys / 32);       // groups of a key warp at most
 constexpr int kScoreSmem = 136 * 1024;               // 1 + 4 + 128.3 KiB at kScoreMaxCap and eight rows a block
+constexpr int kMaxKeysSmem = 200 * 1024;             // 25,600 rows
 // scores and keys, then the inverse norms, the groups and a barrier for each
 __host__ __device__ inline size_t keys_bytes(int n_cap) { return (size_t(n_cap) + 127) / 128 * 128 * 8; }
 __host__ __device__ inline size_t norms_bytes(int n_cap, int r) { return (size_t(n_cap) * r * 4 + 127) / 128 * 128; }
@@ -610,7 +611,7 @@ int launch_cutoff(const actqkv_config* cfg, const Batch& b, const float* scores,
                   int32_t* sel_count, float* budget_real, int32_t* status, cudaStream_t st, const ScoreArgs* score_args = nullptr) {
   if (cfg->thetabar_mode == ACTQKV_THETABAR_ALG1 && (b.layer0 != 0 || b.n_layers != cfg->n_layers))
     return ACTQKV_ERR_UNSUPPORTED;
-  if (size_t(cfg->n_cap) * 8 > 200 * 1024) return ACTQKV_ERR_SHAPE;
+  if (keys_bytes(cfg->n_cap) > kMaxKeysSmem) return ACTQKV_ERR_SHAPE;
   ChainParams p;
   p.scores = scores; p.theta_in = theta_in; p.theta_out = theta_out; p.n_cand = n_cand;
   p.state = static_cast<double*>(budget_state);
@@ -639,10 +640,8 @@ int launch_cutoff(const actqkv_config* cfg, const Batch& b, const float* scores,
   }
   static std::atomic<bool> carved[8][kMaxDevices], opted_in[8][kMaxDevices];
   const int form = score_args ? 4 + 2 * (cfg->head_dim == 128) + (cfg->dtype == ACTQKV_BF16) : 2 * wide + fused;
-  if (sm_sel > 40 * 1024 &&
-      !(score_args ? opt_in_shared_memory(kern, kScoreSmem, opted_in[form])
-                   : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm_sel)) == cudaSuccess))
-    return ACTQKV_ERR_LAUNCH;
+  // one opt-in at the largest size of the form: a size per call could be lowered by another thread ahead of the launch
+  if (sm_sel > 40 * 1024 && !opt_in_shared_memory(kern, score_args ? kScoreSmem : kMaxKeysSmem, opted_in[form])) return ACTQKV_ERR_LAUNCH;
   if (!fused) {
     const size_t sm_chain = sizeof(float) * ((size_t(b.n_layers) * cfg->n_kv_heads + 1) & ~size_t(1)) +
                             sizeof(double) * (2 * size_t(b.n_layers) + 2 * (size_t(cfg->n_layers) + 1));

@@ -141,3 +141,43 @@ def test_scores_taken_by_the_selection(dtype, D, r, n):
             st.step(q, kv, kv, out, advance=False)
             torch.cuda.synchronize()
             assert int(st.status.item()) & B.DEV_TIMEOUT == bit
+
+
+@pytest.mark.parametrize("layers", [1, 2])
+def test_two_threads_with_tables_of_different_size(layers):
+    """Two host threads select from tables of 5,200 and 25,600 rows (the largest): each launch asks for its own amount of
+    shared memory, and neither thread's call may refuse the other's."""
+    import threading
+    import torch
+    from paper_2502_13542_b200 import binding as B
+    spec = wl.llama3_8b_layer().replace(n_layers=layers, k_blocks=16, cap_blocks=16, n_kv_heads=8)
+    done, errors = [], []
+    ready = threading.Barrier(2)
+
+    def work(n):
+        try:
+            cfg, stream = B.make_config(spec, n_cap=n), torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                scores = torch.rand(layers, 8, n, device="cuda")
+                theta = torch.full((layers, 8), 3.0, device="cuda")
+                n_cand = torch.full((1,), n, dtype=torch.int32, device="cuda")
+                state = torch.zeros(1, 1 + 2 * layers, dtype=torch.float64, device="cuda")
+                sel = torch.full((layers, 8, 16), -7, dtype=torch.int32, device="cuda")
+                cnt = torch.zeros(layers, dtype=torch.int32, device="cuda")
+                stream.synchronize()
+                ready.wait()
+                for _ in range(1000):
+                    B.select_cutoff(cfg, B.Batch(1, layers, 0), scores, theta, n_cand, state, sel, cnt, stream=stream)
+                stream.synchronize()
+            k = int(cnt[0])
+            assert sel[0, 0, :k].tolist() == pick(scores[0, 0].tolist(), k)
+            done.append(n)
+        except Exception as e:                            # noqa: BLE001  (handed to the test's thread)
+            errors.append((n, e))
+
+    threads = [threading.Thread(target=work, args=(n,)) for n in (5200, 25600)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors and sorted(done) == [5200, 25600]
