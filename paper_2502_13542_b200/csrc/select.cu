@@ -246,7 +246,7 @@ __device__ __forceinline__ bool wait_phase0(uint32_t bar, uint32_t polls) {
 // an input written by cutoff_chain_kernel.
 //
 // A chain of short phases on the critical path of a step, once per launch.  kKeys threads hold the keys, one warp
-// behind them (control) the chain: the key warps fetch the scores and leave one (maximum, Z, sum e x) per warp; control
+// behind them (control) the chain: the key warps fetch the scores and leave one (maximum, Z, sum e x) per slot; control
 // merges these into the head's density, hands it to the cluster's CTAs by asynchronous remote stores that complete on
 // their barriers, adds up theirs and grants the count in fp64.  Meanwhile the key warps rank their keys against all
 // others, which needs no count; with the count a key is taken if its rank is below it, and one scan over the warps'
@@ -291,7 +291,10 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
   __shared__ int warp_tot[2][kWarps];
   __shared__ float sh_thetas[2][8];            // the densities of the cluster's heads (written by their CTAs), one set per pass
   __shared__ __align__(8) uint64_t sh_bar[2];  // a pass's densities have arrived
-  __shared__ float red_m[kWarps], red_z[kWarps], red_e[kWarps];
+  // Eq. 11 is summed in 16 slots, the scores i = 32 v .. 32 v + 31 (mod 512) in slot v, a slot per warp or two, so that a
+  // density does not depend on the number of key threads, which goes by the size of the batch.
+  constexpr int kSlots = 16, kCols = kKeys == 256 && D == 0 ? 2 : 1;      // (the scoring form has 128 scores at most)
+  __shared__ float red_m[kSlots], red_z[kSlots], red_e[kSlots];
   __shared__ int sh_count, sh_late;            // the granted count; a wait ran out
   const int g = blockIdx.x, unit = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool control = warp == kWarps;
@@ -418,7 +421,8 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
         key_sync<kKeys>();                       // the scores are complete
       }
       // the scores are fetched once, by all threads at a time; density and selection read them from here
-      float m = -INFINITY;
+      float m[2] = {-INFINITY, -INFINITY};       // per column of key threads
+      static_assert(kCols == 1 || kKeys * kCols == 32 * kSlots, "every second fetch is of the other slot");
       for (int i0 = tid; i0 < 4 * n4; i0 += 4 * kKeys) {
         float x[4];
 #pragma unroll
@@ -432,23 +436,26 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
           if (u > 0 && i >= 4 * n4) break;
           if (kFused && i < n) {
             if (D == 0) sc[i] = x[u];
-            m = fmaxf(m, ch.beta * x[u]);
+            m[u & (kCols - 1)] = fmaxf(m[u & (kCols - 1)], ch.beta * x[u]);
           }
           keys[i] = i < n ? score_key(x[u]) : 0u;
         }
       }
-      if (kFused && warp * 32 < n) {           // Eq. 11 over this warp's scores, about the warp's own maximum
-        m = warp_max_redux(m);
-        float z = 0.f, e_x = 0.f;
+      if constexpr (kFused) {                  // Eq. 11 over a slot's scores, about the slot's own maximum
+#pragma unroll 1
+        for (int col = 0; col < kCols && (warp + col * kWarps) * 32 < n; ++col) {
+          const float top = warp_max_redux(col ? m[1] : m[0]);
+          float z = 0.f, e_x = 0.f;
 #pragma unroll 2
-        for (int i = tid; i < n; i += kKeys) {
-          const float x = ch.beta * sc[i] - m, e = expf(x);
-          z += e;
-          e_x = fmaf(e, x, e_x);
+          for (int i = tid + col * kKeys; i < n; i += kKeys * kCols) {
+            const float x = fmaf(ch.beta, sc[i], -top), e = expf(x);
+            z += e;
+            e_x = fmaf(e, x, e_x);
+          }
+          z = warp_sum(z);
+          e_x = warp_sum(e_x);
+          if (lane == 0) { red_m[warp + col * kWarps] = top; red_z[warp + col * kWarps] = z; red_e[warp + col * kWarps] = e_x; }
         }
-        z = warp_sum(z);
-        e_x = warp_sum(e_x);
-        if (lane == 0) { red_m[warp] = m; red_z[warp] = z; red_e[warp] = e_x; }
       }
     } else if constexpr (kFused) {
       // The old state: the mean densities of the deeper layers that have a history (a lane per layer, then a
@@ -473,8 +480,8 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
       float th_own;
       if (ch.theta_in && real) {
         th_own = ch.theta_in[uh];
-      } else {                                 // the warps' sums, moved to the common maximum
-        const bool on = lane < kWarps && lane * 32 < n;
+      } else {                                 // the slots' sums, moved to the common maximum
+        const bool on = lane < kSlots && lane * 32 < n;
         const float m = on ? red_m[lane] : -INFINITY, top = warp_max_redux(m);
         const float x = on ? m - top : 0.f, f = on ? expf(x) : 0.f, zw = on ? red_z[lane] : 0.f;
         float z = f * zw, e_x = on ? f * fmaf(zw, x, red_e[lane]) : 0.f;

@@ -83,6 +83,38 @@ def test_density_and_selection_of_one_layer(seqs, n):
                 assert sel[u, g].tolist() == pick(scores[u, g, :m].tolist(), k) + [-1] * (c - k)
 
 
+@pytest.mark.parametrize("n", [256, 257, 300, 511, 512, 513, 769, 1023, 1500])
+def test_density_does_not_depend_on_the_batch(n):
+    """A sequence's density, count, set and budget are the same bits alone, beside 8 others and beside 11 others (up to 9
+    sequences of 8 heads have 512 key threads where there are more than 256 candidates, more of them have 256)."""
+    import torch
+    from paper_2502_13542_b200 import binding as B
+    L, c = 2, 24
+    spec = wl.llama3_8b_layer().replace(n_layers=L, k_blocks=c, cap_blocks=2 * c, n_kv_heads=8)
+    cfg = B.make_config(spec, n_cap=n, beta=6.0)
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    table = torch.randn(12, 8, n, 4, 128, device="cuda", generator=gen).bfloat16()
+    norms = 1.0 / table.float().norm(dim=-1)
+    probe = torch.randn(12, 8, 128, device="cuda", generator=gen)
+    n_cand = torch.full((12,), n, dtype=torch.int32, device="cuda")
+    n_cand[1] = n - 7
+
+    def run(seqs):
+        scores, theta = torch.zeros(seqs, 8, n, device="cuda"), torch.zeros(seqs, 8, device="cuda")
+        sel, cnt = torch.zeros(seqs, 8, 2 * c, dtype=torch.int32, device="cuda"), torch.zeros(seqs, dtype=torch.int32, device="cuda")
+        state = torch.zeros(seqs, 1 + 2 * L, dtype=torch.float64, device="cuda")
+        for layer in range(L):
+            B.score_select(cfg, B.Batch(seqs, 1, layer), probe[:seqs].contiguous(), table[:seqs].contiguous(),
+                           norms[:seqs].contiguous(), n_cand[:seqs].contiguous(), state, scores, theta, sel, cnt)
+        torch.cuda.synchronize()
+        return scores, theta, sel, cnt, state
+
+    many = run(12)
+    for seqs in (1, 9):
+        for i, (x, y) in enumerate(zip(run(seqs), many)):
+            assert torch.equal(x, y[:seqs]), (seqs, i)
+
+
 @pytest.mark.parametrize("dtype,D,r", [("bf16", 128, 4), ("bf16", 64, 8), ("f32", 128, 2), ("f32", 64, 4)])
 @pytest.mark.parametrize("n", [0, 1, 3, 31, 32, 33, 65, 127, 128, 129])
 def test_scores_taken_by_the_selection(dtype, D, r, n):
