@@ -102,7 +102,7 @@ int launch_attention_tc4(const actqkv_config* cfg, const Batch& b, const AttnArg
 // Prefill windows of any length and group size: two query tiles per CTA; split_p: P in two bf16 terms
 // instead of fp16.
 bool attention_prefill_supported(const actqkv_config* cfg);
-// CTAs of that launch (the CTAs of a cluster that share a key stream counted each).
+// The key streams of that launch times the CTAs that share one (a thin last round of several has a few CTAs more).
 int64_t attention_prefill_ctas(const actqkv_config* cfg, const Batch& b, int n_tokens);
 bool attention_prefill_cuts(const actqkv_config* cfg, const Batch& b, int n_tokens);      // a key stream goes to several CTAs
 int launch_attention_prefill(const actqkv_config* cfg, const Batch& b, const AttnArgs& a, bool split_p, cudaStream_t st);

@@ -28,14 +28,65 @@ LOCAL_CASES = [  # ..., local past
 ]
 
 
-# More streams than SMs: the first 148 (or 296) whole, the rest cut in two as long as they are at most 74; both forms of P.
+# More streams than SMs: behind the first 148 (or 296) at most 74 are left, whose query tiles take a CTA each from 1,024 keys on
+# (not one tile of 40 tokens, nor 300 and 430 keys; 300 tokens at G = 1 are three tiles, a last pair of one); both forms of P.
 ROUND_CASES = [(8, 8, 20, 129, 1501, 16, 512), (16, 8, 20, 128, 1408, 16, 512), (8, 8, 27, 40, 2003, 32, 1024), (8, 8, 28, 40, 2003, 32, 1024),
-               (1, 1, 149, 200, 999, 16, 256), (16, 8, 37, 256, 1152, 16, 256), (24, 8, 46, 41, 801, 16, 0)]
+               (1, 1, 149, 200, 999, 16, 256), (16, 8, 37, 256, 1152, 16, 256), (24, 8, 46, 41, 801, 16, 0), (8, 8, 20, 300, 0, 16, 512), (8, 8, 10, 300, 130, 16, 512),
+               (8, 8, 10, 300, 1500, 16, 512), (24, 8, 46, 83, 1701, 32, 256), (16, 8, 28, 200, 1777, 16, 0)]
 
 
 @pytest.mark.parametrize("hq,hkv,units,nt,past,page,local", ROUND_CASES)
 def test_thin_last_round(hq, hkv, units, nt, past, page, local):
     check(hq, hkv, units, nt, past, page, local, bf16=True)      # (fp32 results of ragged steps are the general kernel's)
+
+
+def test_thin_last_round_of_whole_tiles_fp32_results():
+    check(16, 8, 20, 256, 1408, 16, 512)
+
+
+@pytest.mark.parametrize("hq,hkv,units,layers,nt,past,f32", [
+    (8, 8, 20, 1, 129, 1501, False), (16, 8, 20, 2, 256, 1408, False), (16, 8, 20, 1, 256, 1408, True), (32, 8, 20, 2, 60, 2200, False),
+    (8, 8, 20, 2, 300, 1200, False), (32, 8, 8, 1, 500, 900, False), (32, 8, 8, 4, 512, 900, False), (24, 8, 44, 2, 83, 0, False), (24, 8, 44, 2, 83, 1700, False)])
+def test_results_do_not_depend_on_the_place(hq, hkv, units, layers, nt, past, f32):
+    """Equal sequences (and layers) in one call of more streams than SMs: the bits of every one are those of the first, and of a
+    call of half of them, whose streams are fewer but not cut either (75 and more)."""
+    import torch
+    from paper_2502_13542_b200 import binding as B
+    spec = wl.llama3_8b_layer().replace(n_layers=layers, n_q_heads=hq, n_kv_heads=hkv, k_blocks=9, cap_blocks=9, context=past + nt)
+    per = -(-(past + nt) // 16) + 1
+    cfg = B.make_config(spec, out_dtype=B.F32 if f32 else B.BF16, n_phys_pages=per, max_pages=per)
+    gen = torch.Generator(device="cuda").manual_seed(nt)
+
+    def rnd(*shape):
+        x = torch.randn(*shape, 128, device="cuda", generator=gen)
+        x[..., :3] *= 10.0
+        return x.to(torch.bfloat16)
+
+    table = torch.randperm(per, dtype=torch.int32)
+    pages = [rnd(1, per, hkv, 16).expand(layers, -1, -1, -1, -1).contiguous() for _ in range(2)]
+    step = [rnd(1, nt, h) for h in (hq, hkv, hkv)]
+    n = B.n_candidates(cfg, past) if past > spec.n_init else 0
+    c = min(9, n)
+    sel = torch.stack([torch.randperm(n)[:c].sort().values for _ in range(hkv)]).to(torch.int32)
+
+    def run(units):
+        st = B.RetrievalState(cfg, n_seq=units // layers, n_layers=layers, page_table=table.repeat(units // layers, 1), shared_pages=pages)
+        st.set_positions([past])
+        st.sel_idx[:, :, :c] = sel.cuda()
+        st.sel_count.fill_(c)
+        q, k, v = (x.expand(units, -1, -1, -1).contiguous() for x in step)
+        out = torch.full(q.shape, float("nan"), dtype=cfg.torch_out_dtype, device="cuda")
+        lse = torch.full((units, hq, nt), float("nan"), device="cuda")
+        B.retrieval_attention(cfg, st.batch, q, k, v, nt, st.k_pages, st.v_pages, st.page_table, st.pos0, st.sel_idx, st.sel_count,
+                              out, lse, st.status)
+        torch.cuda.synchronize()
+        assert int(st.status.item()) == 0 and torch.isfinite(out).all()
+        return out, lse
+
+    small, small_lse = run(units // 2)
+    out, lse = run(units)
+    for u in range(units):
+        assert torch.equal(out[u], small[0]) and torch.equal(lse[u], small_lse[0]), u
 
 
 @pytest.mark.parametrize("hq,hkv,units,nt,past,page,local", LOCAL_CASES)
