@@ -4,20 +4,28 @@
 // dim / page size / alignment; serves fp32 caches and what the tensor-core kernels do not take.
 //
 // One CTA = 32 rows of one KV head: the (token, query head) pairs of the group, row = token * G + head,
-// so that K and V are read once per group.  Keys go through shared memory in chunks, as fp32, two buffers: a producer
+// so that K and V are read once per group.  Keys go through shared memory in chunks, as they come, two buffers: a producer
 // warp looks the keys up (position -> page table, behind the selection's entries), brings chunk c + 1 and waits for it while
 // the four compute warps work on chunk c; one CTA barrier per chunk.
-// A compute warp has 8 rows; its lanes have one key each (two at D = 64) in Q K^T and D / 32 channels each in P V.  Bound
-// by the shared-memory bandwidth: Q and P are read by broadcast, one 128-byte wavefront per 16-byte load, and K and V
-// by 32 lanes apart, 16 wavefronts per 64 FMAs of a warp (with 4 rows x 4 keys per thread, 16 lanes to a row, it was 32).
+// A compute warp has 8 rows; its lanes have one or two keys each in Q K^T (one: fp32 at D = 128) and D / 32 channels each in P V.
+// Bound by the shared-memory bandwidth: Q and P are read by broadcast, one 128-byte wavefront per 16-byte load, K and V by 32
+// lanes apart.  Wavefronts per 64 FMAs of a warp, Q K^T and P V: fp32 16 and 16 at D = 64, 24 and 12 at D = 128; bf16, which is
+// unpacked at its use (8 rows share that), 12 and 12, 12 and 8.  (4 rows x 4 keys per thread, 16 lanes to a row: 32.)
 //
 // The initial tokens, the local past and the step's own tokens come first and the selected blocks last: the former are
 // known before this step's selection exists, so their chunks run ahead of the dependency wait (programmatic dependent
 // launch).  Few tiles: the chunks are cut over the CTAs of a cluster (chunk c goes to rank c % n) and the partial
 // results are merged through distributed shared memory.
-// A window of 256 tokens x 4 heads over 1,400 keys (D = 64, fp32), launches one behind the other: 28.7 us with all threads
-// staging each chunk between two barriers and every key behind the wait, 22.3 us like this (25.3 us with a producer lane
-// per 16 bytes, which spent 6k clk a chunk on addresses); a prompt of 16 such windows 663 -> 565 us.
+// Launches one behind the other, us, 4 x 4 tiles with all 128 threads staging fp32 between two barriers and every key behind the
+// wait -> this (one producer warp that unpacks bf16 into fp32, as it was at first, in brackets):
+//                                            fp32 D = 64     fp32 D = 128    bf16 D = 64              bf16 D = 128
+//   1 token, 32 / 8 heads, 4,096 behind        17 ->  13        27 ->  19       17 ->   13  (15)         27 ->   18  (22)
+//   256 tokens, 4 / 2 heads, 1,472 behind      29 ->  22        39 ->  35       29 ->   21  (24)         37 ->   31  (38)
+//   256 tokens, 32 / 8 heads, 1,472 behind    161 ->  99       224 -> 200      166 ->   97 (111)        217 ->  160 (227)
+//   16 sequences of that                    1,492 -> 1,405   2,983 -> 2,837  1,487 -> 1,371 (1,586)   2,839 -> 2,267 (3,197)
+//   64 sequences of 1 token, 1,472 behind     286 -> 180       442 -> 359      290 ->  176 (221)        397 ->  290 (410)
+// An SM holds two of these CTAs where it held four at D = 64: grids that leave some SMs one and some two (80 to 100, 180 to 200 and
+// 320 CTAs) are 1 to 8 % slower in fp32 at D = 64 (45 -> 48, 88 -> 93, 174 -> 182), the ones beside them up to 1.8 times as fast.
 #include <algorithm>
 #include <type_traits>
 
@@ -33,13 +41,13 @@ constexpr int kComputeWarps = 4, kRowsPerWarp = kRows / kComputeWarps;
 constexpr int kThreads = 32 * (kComputeWarps + 1);
 constexpr int kMaxSplits = 8;
 
-template <int D> struct Smem {
-  static constexpr int kChunk = D == 64 ? 64 : 32;   // keys; two CTAs per SM
-  static constexpr int kKStride = D + 4;             // floats; 32 consecutive keys at one channel vector hit distinct banks
-  static constexpr int kPStride = kChunk + 4;
-  static constexpr int kKV = kChunk * (kKStride + D);                   // one buffer: K, then V
-  static constexpr int kQ = 0, kBuf = kQ + kRows * D, kP = kBuf + 2 * kKV, kFloats = kP + kRows * kPStride;
-  static constexpr int kBytes = kFloats * 4;
+// Bytes.  K and V lie there as they come (bf16 is unpacked at its use), Q and P as fp32.
+template <typename T, int D> struct Smem {
+  static constexpr int kChunk = D * sizeof(T) > 256 ? 32 : 64;          // keys; two CTAs per SM
+  static constexpr int kKStride = D + Vec16<T>::N;   // elements; 8 consecutive keys at one 16-byte vector hit distinct banks
+  static constexpr int kPStride = kChunk + 4;        // floats
+  static constexpr int kKV = kChunk * (kKStride + D) * int(sizeof(T));  // one buffer: K, then V
+  static constexpr int kQ = 0, kBuf = kQ + kRows * D * 4, kP = kBuf + 2 * kKV, kBytes = kP + kRows * kPStride * 4;
 };
 
 struct SimtParams {
@@ -72,17 +80,17 @@ __device__ __forceinline__ float ld_peer(const float* local, uint32_t rank) {
   asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
   return v;
 }
-__device__ __forceinline__ void cp_async16(float* dst, const void* src) {
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(uint32_t(__cvta_generic_to_shared(dst))), "l"(src) : "memory");
 }
 
 template <typename T, typename TO, int D>
 __global__ void __launch_bounds__(kThreads, 2) attention_simt_kernel(SimtParams p) {
-  using S = Smem<D>;
+  using S = Smem<T, D>;
   constexpr int kChunk = S::kChunk, KPL = kChunk / 32, CPL = D / 32;   // keys and channels per lane
   constexpr int VN = Vec16<T>::N, VPR = D / VN, R = kRowsPerWarp;
-  extern __shared__ __align__(16) float sm[];
-  float *Qs = sm + S::kQ, *Ps = sm + S::kP;
+  extern __shared__ __align__(16) unsigned char sm[];
+  float *Qs = reinterpret_cast<float*>(sm + S::kQ), *Ps = reinterpret_cast<float*>(sm + S::kP);
   __shared__ float part_m[kRows], part_l[kRows];
 
   grid_launch_dependents();          // the append makes its loads while this kernel runs
@@ -179,8 +187,8 @@ __global__ void __launch_bounds__(kThreads, 2) attention_simt_kernel(SimtParams 
       return x;
     };
     // Two lanes per key, 16 keys at a time: whole 32-byte sectors, and no address arithmetic between a row's copies.
-    auto bring = [&](int64_t c, const Places& x, float* Ks) {
-      float* Vs = Ks + kChunk * S::kKStride;
+    auto bring = [&](int64_t c, const Places& x, T* Ks) {
+      T* Vs = Ks + kChunk * S::kKStride;
       const int half = lane & 1;
 #pragma unroll
       for (int j = 0; j < 2 * KPL; ++j) {
@@ -188,41 +196,16 @@ __global__ void __launch_bounds__(kThreads, 2) attention_simt_kernel(SimtParams 
         const int64_t at = __shfl_sync(0xffffffffu, x.at[j >> 1], in);
         const bool past = c >= early || c * kChunk + row < n_past;
         const T *ks = (past ? kp : kw) + at + half * VN, *vs = (past ? vp : vw) + at + half * VN;
-        float *kd = Ks + row * S::kKStride + half * VN, *vd = Vs + row * D + half * VN;
+        T *kd = Ks + row * S::kKStride + half * VN, *vd = Vs + row * D + half * VN;
         if (at < 0) {
 #pragma unroll 1
           for (int e = 0; e < D; e += 2 * VN)
-#pragma unroll
-            for (int f = 0; f < VN; f += 4)
-              *reinterpret_cast<float4*>(kd + e + f) = *reinterpret_cast<float4*>(vd + e + f) = make_float4(0.f, 0.f, 0.f, 0.f);
-        } else if constexpr (sizeof(T) == 4) {
+            *reinterpret_cast<uint4*>(kd + e) = *reinterpret_cast<uint4*>(vd + e) = make_uint4(0, 0, 0, 0);
+        } else {
 #pragma unroll
           for (int e = 0; e < D; e += 2 * VN) {
             cp_async16(kd + e, ks + e);
             cp_async16(vd + e, vs + e);
-          }
-        } else {
-          constexpr int kBatch = 4;
-#pragma unroll
-          for (int e0 = 0; e0 < D; e0 += 2 * VN * kBatch) {
-            uint4 kr[kBatch], vr[kBatch];
-#pragma unroll
-            for (int u = 0; u < kBatch; ++u) {
-              kr[u] = __ldg(reinterpret_cast<const uint4*>(ks + e0 + u * 2 * VN));
-              vr[u] = __ldg(reinterpret_cast<const uint4*>(vs + e0 + u * 2 * VN));
-            }
-#pragma unroll
-            for (int u = 0; u < kBatch; ++u) {
-              float kf[VN], vf[VN];
-              Vec16<T>::unpack(kr[u], kf);
-              Vec16<T>::unpack(vr[u], vf);
-#pragma unroll
-              for (int f = 0; f < VN; f += 4) {
-                const int e = e0 + u * 2 * VN + f;
-                *reinterpret_cast<float4*>(kd + e) = make_float4(kf[f], kf[f + 1], kf[f + 2], kf[f + 3]);
-                *reinterpret_cast<float4*>(vd + e) = make_float4(vf[f], vf[f + 1], vf[f + 2], vf[f + 3]);
-              }
-            }
           }
         }
       }
@@ -231,7 +214,7 @@ __global__ void __launch_bounds__(kThreads, 2) attention_simt_kernel(SimtParams 
     if (c >= early) wait_selection();
     Places x = look_up(c);
     for (int buf = 0; c < total; buf ^= 1) {
-      bring(c, x, sm + S::kBuf + buf * S::kKV);
+      bring(c, x, reinterpret_cast<T*>(sm + S::kBuf + buf * S::kKV));
       c += p.n_splits;
       const bool known = c < early || open;
       if (known && c < total) x = look_up(c);          // while the copies fly
@@ -254,7 +237,7 @@ __global__ void __launch_bounds__(kThreads, 2) attention_simt_kernel(SimtParams 
       if (c >= early && !open) wait_selection();
       if (c >= total) break;
       __syncthreads();                                 // the chunk is there
-      const float *Ks = sm + S::kBuf + buf * S::kKV, *Vs = Ks + kChunk * S::kKStride;
+      const T *Ks = reinterpret_cast<const T*>(sm + S::kBuf + buf * S::kKV), *Vs = Ks + kChunk * S::kKStride;
       // ---- S = Q K^T: keys lane + 32 j
       float s[R][KPL];
 #pragma unroll
@@ -262,20 +245,22 @@ __global__ void __launch_bounds__(kThreads, 2) attention_simt_kernel(SimtParams 
 #pragma unroll
         for (int j = 0; j < KPL; ++j) s[r][j] = 0.f;
 #pragma unroll 2
-      for (int d = 0; d < D; d += 4) {
-        float4 kv[KPL], qv[R];
+      for (int d = 0; d < D; d += VN) {
+        float kv[KPL][VN];
 #pragma unroll
-        for (int j = 0; j < KPL; ++j) kv[j] = *reinterpret_cast<const float4*>(Ks + (lane + 32 * j) * S::kKStride + d);
-#pragma unroll
-        for (int r = 0; r < R; ++r) qv[r] = *reinterpret_cast<const float4*>(q_rows + r * D + d);
+        for (int j = 0; j < KPL; ++j) Vec16<T>::load(Ks + (lane + 32 * j) * S::kKStride + d, kv[j]);
 #pragma unroll
         for (int r = 0; r < R; ++r)
 #pragma unroll
-          for (int j = 0; j < KPL; ++j) {
-            s[r][j] = fmaf(qv[r].x, kv[j].x, s[r][j]);
-            s[r][j] = fmaf(qv[r].y, kv[j].y, s[r][j]);
-            s[r][j] = fmaf(qv[r].z, kv[j].z, s[r][j]);
-            s[r][j] = fmaf(qv[r].w, kv[j].w, s[r][j]);
+          for (int e = 0; e < VN; e += 4) {
+            const float4 qv = *reinterpret_cast<const float4*>(q_rows + r * D + d + e);
+#pragma unroll
+            for (int j = 0; j < KPL; ++j) {
+              s[r][j] = fmaf(qv.x, kv[j][e], s[r][j]);
+              s[r][j] = fmaf(qv.y, kv[j][e + 1], s[r][j]);
+              s[r][j] = fmaf(qv.z, kv[j][e + 2], s[r][j]);
+              s[r][j] = fmaf(qv.w, kv[j][e + 3], s[r][j]);
+            }
           }
       }
       // ---- running softmax of the warp's rows
@@ -316,7 +301,20 @@ __global__ void __launch_bounds__(kThreads, 2) attention_simt_kernel(SimtParams 
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
           float v[CPL];
-          if constexpr (CPL == 2) {
+          if constexpr (sizeof(T) == 2) {              // bf16 is the upper half of an fp32
+            uint32_t raw[CPL / 2];
+            if constexpr (CPL == 2) {
+              raw[0] = *reinterpret_cast<const uint32_t*>(Vs + (k + kk) * D + 2 * lane);
+            } else {
+              const uint2 t = *reinterpret_cast<const uint2*>(Vs + (k + kk) * D + 4 * lane);
+              raw[0] = t.x; raw[1] = t.y;
+            }
+#pragma unroll
+            for (int q = 0; q < CPL / 2; ++q) {
+              v[2 * q] = __uint_as_float(raw[q] << 16);
+              v[2 * q + 1] = __uint_as_float(raw[q] & 0xFFFF0000u);
+            }
+          } else if constexpr (CPL == 2) {
             const float2 t = *reinterpret_cast<const float2*>(Vs + (k + kk) * D + 2 * lane);
             v[0] = t.x; v[1] = t.y;
           } else {
@@ -419,13 +417,14 @@ template <typename T, typename TO, int D>
 int launch(const SimtParams& p, dim3 grid, cudaStream_t st) {
   static std::atomic<bool> opted_in[kMaxDevices];
   auto kern = attention_simt_kernel<T, TO, D>;
-  if (!opt_in_shared_memory(kern, Smem<D>::kBytes, opted_in)) return ACTQKV_ERR_LAUNCH;
+  constexpr int kBytes = Smem<T, D>::kBytes;
+  if (!opt_in_shared_memory(kern, kBytes, opted_in)) return ACTQKV_ERR_LAUNCH;
   static std::atomic<bool> carved[kMaxDevices];
   prefer_max_shared(kern, carved);
   cudaLaunchConfig_t lc = {};
   lc.gridDim = grid;
   lc.blockDim = dim3(kThreads, 1, 1);
-  lc.dynamicSmemBytes = Smem<D>::kBytes;
+  lc.dynamicSmemBytes = kBytes;
   lc.stream = st;
   cudaLaunchAttribute attr[2];
   allow_early_launch(attr[0]);

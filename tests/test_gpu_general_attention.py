@@ -87,7 +87,8 @@ def test_general_attention_against_fp64(dtype, D, hq, hkv, units, nt, past, page
 # behind it; fewer of them than ranks; several rows per lane group and rows past the last token.
 EARLY_EDGES = [("f32", 64, 4, 2, 1, nt, past, 16, 0) for nt in (63, 64, 65) for past in (704, 705)] + [
     ("f32", 64, 4, 2, 40, 16, 832, 16, 0), ("f32", 128, 4, 1, 1, 31, 897, 16, 0), ("f32", 128, 4, 1, 1, 32, 768, 16, 0),
-    ("bf16", 64, 8, 2, 1, 127, 761, 16, 8), ("bf16", 128, 2, 1, 2, 33, 831, 16, 0), ("bf16", 64, 2, 2, 1, 1, 704, 16, 0)]
+    ("bf16", 64, 8, 2, 1, 127, 761, 16, 8), ("bf16", 128, 2, 1, 2, 33, 831, 16, 0), ("bf16", 64, 2, 2, 1, 1, 704, 16, 0)] + [
+    ("bf16", 128, hq, 2, 2, nt, past, 16, 0) for hq, nt, past in ((4, 63, 704), (4, 64, 704), (6, 65, 705), (2, 1, 769), (16, 31, 737))]
 
 
 @pytest.mark.parametrize("dtype,D,hq,hkv,units,nt,past,page,local", EARLY_EDGES)
