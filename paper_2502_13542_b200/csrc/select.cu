@@ -6,13 +6,14 @@
 //                        the layers shallow -> deep in fp64: B^l from Eq. 12, the granted
 //                        integer c^l, the running B_kv and the density history.
 //   select_kernel        one CTA per (unit, KV head).  Scores become order-preserving 32-bit
-//                        keys in shared memory; up to 384 keys are ranked against one another, of more the
-//                        c-th largest is found by a search on the bits; equal keys are admitted lowest index
-//                        first; the survivors are compacted in ascending block order.
+//                        keys in shared memory; up to 384 keys (256 where 256 threads hold
+//                        them) are ranked against one another, of more the c-th largest is found
+//                        by a search on the bits; equal keys are admitted lowest index first; the
+//                        survivors are compacted in ascending block order.
 // A call for one layer (the usual layer-by-layer use) runs select_kernel alone: the Hkv CTAs of a
 // sequence form a thread-block cluster, each takes its head's density, they exchange the values
 // through distributed shared memory, every CTA evaluates Eq. 12 for itself and the first one
-// writes the budget state back.  Where the table is small it takes the scores, too.
+// writes the budget state back.  Behind bias + probe of a window it takes the scores of a small table, too.
 #include "common.cuh"
 #include "stages.cuh"
 
@@ -250,7 +251,7 @@ __device__ __forceinline__ bool wait_phase0(uint32_t bar, uint32_t polls) {
 // merges these into the head's density, hands it to the cluster's CTAs by asynchronous remote stores that complete on
 // their barriers, adds up theirs and grants the count in fp64.  Meanwhile the key warps rank their keys against all
 // others, which needs no count; with the count a key is taken if its rank is below it, and one scan over the warps'
-// ballots places it.  Beyond kRankMax candidates the n^2 comparisons are longer than the chain beside them, and the
+// ballots places it.  Beyond kRankMax candidates (or a key per thread) the n^2 comparisons are longer than the chain beside them, and the
 // c-th largest key is found instead by a search on its bits (a threshold per warp and step), which ends as soon as a
 // threshold separates exactly c keys.  Score and selection of one layer, 60 of these pairs chained in a graph, us per pair
 // at 128 / 251 / 313 / 384 / 450 / 512 candidates: ranks 4.6 / 5.6 / 6.2 / 7.0 / 8.2 / 8.7, search 5.9 / 6.0 / 6.6 / 6.8 / 6.9 /
@@ -281,7 +282,8 @@ __host__ __device__ inline size_t keys_bytes(int n_cap) { return (size_t(n_cap) 
 __host__ __device__ inline size_t norms_bytes(int n_cap, int r) { return (size_t(n_cap) * r * 4 + 127) / 128 * 128; }
 __host__ __device__ inline int slots_of(int n_cap) { return (n_cap + 4 * (kScoreKeys / 32) - 1) / (4 * (kScoreKeys / 32)); }
 
-template <bool kFused, int kKeys, typename T, int D>
+// kCols: slots of the density that a key warp sums.
+template <bool kFused, int kKeys, int kCols, typename T, int D>
 __global__ void __launch_bounds__(kKeys + 32)
 select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_cand,
               int32_t* __restrict__ sel_count, int32_t* __restrict__ sel_idx, int n_kv_heads,
@@ -291,9 +293,9 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
   __shared__ int warp_tot[2][kWarps];
   __shared__ float sh_thetas[2][8];            // the densities of the cluster's heads (written by their CTAs), one set per pass
   __shared__ __align__(8) uint64_t sh_bar[2];  // a pass's densities have arrived
-  // Eq. 11 is summed in 16 slots, the scores i = 32 v .. 32 v + 31 (mod 512) in slot v, a slot per warp or two, so that a
-  // density does not depend on the number of key threads, which goes by the size of the batch.
-  constexpr int kSlots = 16, kCols = kKeys == 256 && D == 0 ? 2 : 1;      // (the scoring form has 128 scores at most)
+  // Eq. 11 is summed in 16 slots, the scores i = 32 v .. 32 v + 31 (mod 512) in slot v, one per warp or two, so that a density
+  // does not depend on the number of key threads, which goes by the size of the batch.  (256 candidates fill 8 slots.)
+  constexpr int kSlots = kWarps * kCols;
   __shared__ float red_m[kSlots], red_z[kSlots], red_e[kSlots];
   __shared__ int sh_count, sh_late;            // the granted count; a wait ran out
   const int g = blockIdx.x, unit = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -422,7 +424,7 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
       }
       // the scores are fetched once, by all threads at a time; density and selection read them from here
       float m[2] = {-INFINITY, -INFINITY};       // per column of key threads
-      static_assert(kCols == 1 || kKeys * kCols == 32 * kSlots, "every second fetch is of the other slot");
+      static_assert(kCols == 1 || (kCols == 2 && kKeys == 256), "every second fetch is of the other slot");
       for (int i0 = tid; i0 < 4 * n4; i0 += 4 * kKeys) {
         float x[4];
 #pragma unroll
@@ -441,21 +443,33 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
           keys[i] = i < n ? score_key(x[u]) : 0u;
         }
       }
-      if constexpr (kFused) {                  // Eq. 11 over a slot's scores, about the slot's own maximum
-#pragma unroll 1
-        for (int col = 0; col < kCols && (warp + col * kWarps) * 32 < n; ++col) {
-          const float top = warp_max_redux(col ? m[1] : m[0]);
-          float z = 0.f, e_x = 0.f;
+      if (kFused && warp * 32 < n) {           // Eq. 11 over a slot's scores, about the slot's own maximum; both slots of a warp at a time
+        float top[kCols], z[kCols], e_x[kCols];
+#pragma unroll
+        for (int col = 0; col < kCols; ++col) { top[col] = warp_max_redux(m[col]); z[col] = e_x[col] = 0.f; }
 #pragma unroll 2
-          for (int i = tid + col * kKeys; i < n; i += kKeys * kCols) {
-            const float x = fmaf(ch.beta, sc[i], -top), e = expf(x);
-            z += e;
-            e_x = fmaf(e, x, e_x);
+        for (int i = tid; i < n; i += kKeys * kCols) {
+#pragma unroll
+          for (int col = 0; col < kCols; ++col) {
+            if (col > 0 && i + col * kKeys >= n) break;
+            const float x = fmaf(ch.beta, sc[i + col * kKeys], -top[col]), e = expf(x);
+            z[col] += e;
+            e_x[col] = fmaf(e, x, e_x[col]);
           }
-          z = warp_sum(z);
-          e_x = warp_sum(e_x);
-          if (lane == 0) { red_m[warp + col * kWarps] = top; red_z[warp + col * kWarps] = z; red_e[warp + col * kWarps] = e_x; }
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+          for (int col = 0; col < kCols; ++col) {
+            z[col] += __shfl_xor_sync(0xffffffffu, z[col], o);
+            e_x[col] += __shfl_xor_sync(0xffffffffu, e_x[col], o);
+          }
+        if (lane == 0)
+#pragma unroll
+          for (int col = 0; col < kCols; ++col) {
+            const int v = warp + col * kWarps;
+            red_m[v] = top[col]; red_z[v] = z[col]; red_e[v] = e_x[col];
+          }
       }
     } else if constexpr (kFused) {
       // The old state: the mean densities of the deeper layers that have a history (a lane per layer, then a
@@ -603,7 +617,8 @@ select_kernel(const float* __restrict__ scores, const int32_t* __restrict__ n_ca
 // a layer at 4 / 40 / 96 candidates: one sequence of 8 KV heads -0.7 to -1.8 / -0.3 to -1.1 / -0.1 to -4.1, two -2.2 to +0.9 / -2.2 to
 // +1.0 / -2.1 to +0.5 (the losses at 64 and 128 tokens), three -2.9 to +0.5 / -2.4 to +3.3 / -3.1 to +5.5, four +0.7 to +2.0 / +1.0 to +4.0 /
 // -0.6 to +2.2; 2 KV heads (fp32) gain up to four sequences.  So it is taken up to 16 heads in all.  At 120 candidates of a table
-// of 128 it is even (-2 to +2.9), but a prompt comes through all the smaller counts first.
+// of 128 it is even (-2 to +2.9), but a prompt comes through all the smaller counts first.  The line goes by the rows of the table,
+// which the host knows, and not by the candidates in it: a prompt in a state sized for more than 16k tokens takes two kernels.
 // Behind anything shorter than bias + probe the copies are exposed (the append of the step before lets nothing start
 // early): a decode step with attention and append takes 14.6 / 17.9 / 18.5 us as two kernels and 15.2 / 19.4 / 20.6 as one at
 // 8 / 40 / 96 candidates, 27.5 and 29.3 with four sequences at 96, a drafted step of 5 tokens 21.0 and 23.9.
@@ -634,19 +649,24 @@ int launch_cutoff(const actqkv_config* cfg, const Batch& b, const float* scores,
   // registers; 16 sequences of 32k-131k tokens, a decode step of two layers: 168 us).
   const bool wide = cfg->n_cap > 256 && b.units() * cfg->n_kv_heads <= kNumSMs / 2;
   using bf16 = __nv_bfloat16;
-  auto kern = fused ? (wide ? select_kernel<true, 512, float, 0> : select_kernel<true, 256, float, 0>)
-                    : (wide ? select_kernel<false, 512, float, 0> : select_kernel<false, 256, float, 0>);
+  // Two slots of the density per warp where 256 threads may have more than 256 scores: 0.2 to 0.5 us a launch (16 sequences at 313 / 500
+  // / 900 candidates 16.0 -> 16.2, 19.7 -> 20.1, 28.5 -> 28.8 with the scores), which smaller tables do not pay.  (The 8 slots of the narrow
+  // form in the wide one, too: 0.3 us on every single sequence above 256.)
+  const bool two_slots = fused && !wide && cfg->n_cap > 256;
+  auto kern = fused ? (wide        ? select_kernel<true, 512, 1, float, 0>
+                       : two_slots ? select_kernel<true, 256, 2, float, 0> : select_kernel<true, 256, 1, float, 0>)
+                    : (wide ? select_kernel<false, 512, 1, float, 0> : select_kernel<false, 256, 1, float, 0>);
   ScoreArgs sa = {};
   size_t sm_sel = keys_bytes(cfg->n_cap);
   if (score_args) {
     sa = *score_args;
     const bool half = cfg->dtype == ACTQKV_BF16;
-    kern = cfg->head_dim == 128 ? (half ? select_kernel<true, kScoreKeys, bf16, 128> : select_kernel<true, kScoreKeys, float, 128>)
-                                : (half ? select_kernel<true, kScoreKeys, bf16, 64> : select_kernel<true, kScoreKeys, float, 64>);
+    kern = cfg->head_dim == 128 ? (half ? select_kernel<true, kScoreKeys, 1, bf16, 128> : select_kernel<true, kScoreKeys, 1, float, 128>)
+                                : (half ? select_kernel<true, kScoreKeys, 1, bf16, 64> : select_kernel<true, kScoreKeys, 1, float, 64>);
     sm_sel += norms_bytes(cfg->n_cap, sa.r) + size_t(kScoreKeys / 32) * (slots_of(cfg->n_cap) * kGroupBytes + kScoreSlots * 8);
   }
-  static std::atomic<bool> carved[8][kMaxDevices], opted_in[8][kMaxDevices];
-  const int form = score_args ? 4 + 2 * (cfg->head_dim == 128) + (cfg->dtype == ACTQKV_BF16) : 2 * wide + fused;
+  static std::atomic<bool> carved[9][kMaxDevices], opted_in[9][kMaxDevices];
+  const int form = score_args ? 4 + 2 * (cfg->head_dim == 128) + (cfg->dtype == ACTQKV_BF16) : two_slots ? 8 : 2 * wide + fused;
   // one opt-in at the largest size of the form: a size per call could be lowered by another thread ahead of the launch
   if (sm_sel > 40 * 1024 && !opt_in_shared_memory(kern, score_args ? kScoreSmem : kMaxKeysSmem, opted_in[form])) return ACTQKV_ERR_LAUNCH;
   if (!fused) {
