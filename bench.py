@@ -90,7 +90,7 @@ class ClockSampler(threading.Thread):
 # DRAM traffic of one launch of the attention kernel (dram__bytes_read.sum + dram__bytes_write.sum of one
 # ncu capture of this workload), valid only for the kernel source it was taken on: the figure is
 # reported while the sha256 of the kernel file still starts with the recorded digits, else null.
-ATTENTION_TRAFFIC = {"source_sha256_16": "aae15457738a9fb3", "bytes_per_launch": 23676416}
+ATTENTION_TRAFFIC = {"source_sha256_16": "bdb6089049063a0d", "bytes_per_launch": 23676672}
 
 
 def attention_traffic():

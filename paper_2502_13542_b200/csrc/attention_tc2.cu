@@ -593,7 +593,9 @@ attention_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
           }
         }
       }
-      if (p.out_bf16) {                                   // whole 128-byte lines, eight lanes to a row (245.2 -> 242.8 us for four layers at 32k)
+      // whole 128-byte lines, eight lanes to a row (four layers at 32k 246.0 -> 243.0 us, 131k 181.0 -> 180.1; runs of one side
+      // 0.1 and 0.3 % apart)
+      if (p.out_bf16) {
         __syncwarp();
         __nv_bfloat16* ob = static_cast<__nv_bfloat16*>(p.a.out) +
                             ((size_t(unit) * nt + size_t(mt) * kBM + q4 * 32) * p.n_q_heads + h) * kD + hw * 64;
