@@ -8,10 +8,11 @@
 // warp looks the keys up (position -> page table, behind the selection's entries), brings chunk c + 1 and waits for it while
 // the four compute warps work on chunk c; one CTA barrier per chunk.
 // A compute warp has 8 rows; its lanes have one or two keys each in Q K^T (one: fp32 at D = 128) and D / 32 channels each in P V.
-// Bound by what two compute warps a scheduler can hide of shared memory and arithmetic (four sequences of 256 tokens, 32 heads: issue slots
-// busy 58 to 71 %, FMA pipe 43 to 55 %, shared memory 54 and 60 % in fp32, 46 and 45 % in bf16).  Q and P are read by broadcast, one
-// 128-byte wavefront per 16-byte load, K and V by 32 lanes apart.  Wavefronts per 64 FMAs of a warp, Q K^T and P V: fp32 16 and 16 at D = 64, 24 and 12 at D = 128; bf16, which is
-// unpacked at its use (8 rows share that), 12 and 12, 12 and 8.  (4 rows x 4 keys per thread, 16 lanes to a row: 32.)
+// Bound by what two compute warps a scheduler can hide of shared memory and arithmetic (four sequences of 256 tokens, 32
+// heads: issue slots busy 58 to 71 %, FMA pipe 43 to 55 %, shared memory 54 and 60 % in fp32, 46 and 45 % in bf16).  Q and P
+// are read by broadcast, one 128-byte wavefront per 16-byte load, K and V by 32 lanes apart.  Wavefronts per 64 FMAs of a warp,
+// Q K^T and P V: fp32 16 and 16 at D = 64, 24 and 12 at D = 128; bf16, which is unpacked at its use (8 rows share that), 12
+// and 12, 12 and 8.  (4 rows x 4 keys per thread, 16 lanes to a row: 32.)
 //
 // The initial tokens, the local past and the step's own tokens come first and the selected blocks last: the former are
 // known before this step's selection exists, so their chunks run ahead of the dependency wait (programmatic dependent
